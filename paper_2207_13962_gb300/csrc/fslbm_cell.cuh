@@ -102,25 +102,55 @@ __device__ __forceinline__ void block_prefix(int n, int* off, F f) {
 }
 
 // ---------------------------------------------------------- cell algebra
+// c_i . (x, y, z) from the components of c_i that are not zero, in the order
+// x, y, z.  Without fast-math the compiler has to keep a product 0 * x and
+// its addition; leaving them out changes no finite value (at most the sign
+// of a zero).
+template <class R>
+__device__ __forceinline__ R cdot(int i, R x, R y, R z) {
+  R s = R(0.0);
+  bool any = false;
+  if (CX(i) != 0) {
+    s = CX(i) > 0 ? x : -x;
+    any = true;
+  }
+  if (CY(i) != 0) {
+    const R v = CY(i) > 0 ? y : -y;
+    s = any ? s + v : v;
+    any = true;
+  }
+  if (CZ(i) != 0) {
+    const R v = CZ(i) > 0 ? z : -z;
+    s = any ? s + v : v;
+  }
+  return s;
+}
+
 // Eq. nm-lbm-equilibrium with c_s^2 = 1/3.
 template <int Q, class R>
 __device__ __forceinline__ R feq_i(int i, R rho, R ux, R uy, R uz) {
-  R cu = R(CX(i)) * ux + R(CY(i)) * uy + R(CZ(i)) * uz;
+  R cu = cdot<R>(i, ux, uy, uz);
   R usq = ux * ux + uy * uy + uz * uz;
   R t = R(1.0) + R(3.0) * cu;
   t = t + R(4.5) * cu * cu;
   t = t - R(1.5) * usq;
   return W<Q, R>(i) * rho * t;
 }
-// Guo source without its (1 - omega/2) factor (Eq. nm-lbm-force-guo).
-template <int Q, class R>
-__device__ __forceinline__ R guo_i(int i, R ux, R uy, R uz, R Fx, R Fy, R Fz) {
-  R cx = R(CX(i)), cy = R(CY(i)), cz = R(CZ(i));
-  R cu = cx * ux + cy * uy + cz * uz;
-  R cF = cx * Fx + cy * Fy + cz * Fz;
-  R uF = ux * Fx + uy * Fy + uz * Fz;
-  R t = R(3.0) * (cF - uF) + R(9.0) * cu * cF;
-  return W<Q, R>(i) * t;
+// f^eq of the pair (i, ibar): cu_ibar = -cu exactly, so the two share every
+// product; each value is that of feq_i.  wr = w_i rho, b = 1.5 u.u.
+template <class R>
+__device__ __forceinline__ void feq_pair(R wr, R cu, R b, R& ei, R& ej) {
+  const R c3 = R(3.0) * cu, a = R(4.5) * cu * cu;
+  ei = wr * (((R(1.0) + c3) + a) - b);
+  ej = wr * (((R(1.0) - c3) + a) - b);
+}
+// Guo source of the pair (i, ibar) without its (1 - omega/2) factor
+// (Eq. nm-lbm-force-guo): w (3 (c.F - u.F) + 9 (c.u)(c.F)).
+template <class R>
+__device__ __forceinline__ void guo_pair(R w, R cu, R cF, R uF, R& si, R& sj) {
+  const R n = R(9.0) * cu * cF;
+  si = w * (R(3.0) * (cF - uF) + n);
+  sj = w * (n - R(3.0) * (cF + uF));
 }
 // rho = sum f (Eq. nm-lbm-density); j sums in direction order.
 template <int Q, class R>
@@ -166,6 +196,13 @@ __device__ __forceinline__ R les_tau(R qxx, R qyy, R qzz, R qxy, R qxz, R qyz, R
 // F = rho g, SRT relaxing towards f^eq, or TRT; with the Smagorinsky model
 // when coll_les(COLL)).  f is overwritten with f*.  Returns rho; sets
 // unstable when |u|^2 >= c_s^2, rho <= 0 or NaN.
+//
+// This is the FP64 engine's collision, bound by the FP64 pipe (two lanes a
+// clock per SM), so it is written to need few FP64 operations while every
+// result keeps the rounding of a per-direction evaluation: the directions i
+// and ibar share c.u, c.F and their products (exact negations), terms with a
+// zero component of c_i are left out, and the factors 1/2 of the symmetric
+// and antisymmetric parts (exact) go into the relaxation rates.
 template <int Q, class R, int COLL>
 __device__ __forceinline__ R collide(R* f, const KParams& p, bool& unstable) {
   R rho, jx, jy, jz;
@@ -178,35 +215,49 @@ __device__ __forceinline__ R collide(R* f, const KParams& p, bool& unstable) {
   R usq = ux * ux + uy * uy + uz * uz;
   if (!(usq < R(1.0 / 3.0)) || !(rho > R(0.0))) unstable = true;
   R omega = R(p.omega);
+  const R b = R(1.5) * usq;
+  const R uF = ux * Fx + uy * Fy + uz * Fz;
+  const R fe0 = (W<Q, R>(0) * rho) * (R(1.0) - b);
   if constexpr (coll_les(COLL)) {
     // momentum flux of the non-equilibrium part, summed in direction order
+    // (the rest direction adds nothing)
     R qxx = R(0.0), qyy = R(0.0), qzz = R(0.0), qxy = R(0.0), qxz = R(0.0), qyz = R(0.0);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const R cx = R(CX(i)), cy = R(CY(i)), cz = R(CZ(i));
-      const R dn = f[i] - feq_i<Q, R>(i, rho, ux, uy, uz);
-      qxx = qxx + cx * cx * dn;
-      qyy = qyy + cy * cy * dn;
-      qzz = qzz + cz * cz * dn;
-      qxy = qxy + cx * cy * dn;
-      qxz = qxz + cx * cz * dn;
-      qyz = qyz + cy * cz * dn;
+    for (int i = 1; i < Q; i += 2) {
+      const R cu = cdot<R>(i, ux, uy, uz);
+      R e[2];
+      feq_pair<R>(W<Q, R>(i) * rho, cu, b, e[0], e[1]);
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {  // c_a c_b is the same for i and ibar
+        const R dn = f[i + k] - e[k];
+        if (CX(i) != 0) qxx = qxx + dn;
+        if (CY(i) != 0) qyy = qyy + dn;
+        if (CZ(i) != 0) qzz = qzz + dn;
+        if (CX(i) * CY(i) != 0) qxy = CX(i) * CY(i) > 0 ? qxy + dn : qxy - dn;
+        if (CX(i) * CZ(i) != 0) qxz = CX(i) * CZ(i) > 0 ? qxz + dn : qxz - dn;
+        if (CY(i) * CZ(i) != 0) qyz = CY(i) * CZ(i) > 0 ? qyz + dn : qyz - dn;
+      }
     }
     omega = R(1.0) / les_tau<R>(qxx, qyy, qzz, qxy, qxz, qyz, rho, omega, R(p.cs));
   }
+  const R s0 = W<Q, R>(0) * (R(3.0) * (-uF));
   if constexpr (!coll_trt(COLL)) {
     const R om = omega, pref = coll_les(COLL) ? R(1.0) - R(0.5) * omega : R(p.pref_p);
+    f[0] = f[0] - om * (f[0] - fe0) + pref * s0;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      R fe = feq_i<Q, R>(i, rho, ux, uy, uz);
-      R s = guo_i<Q, R>(i, ux, uy, uz, Fx, Fy, Fz);
-      f[i] = f[i] - om * (f[i] - fe) + pref * s;
+    for (int i = 1; i < Q; i += 2) {
+      const int j = i + 1;
+      const R cu = cdot<R>(i, ux, uy, uz), cF = cdot<R>(i, Fx, Fy, Fz);
+      R ei, ej, si, sj;
+      feq_pair<R>(W<Q, R>(i) * rho, cu, b, ei, ej);
+      guo_pair<R>(W<Q, R>(i), cu, cF, uF, si, sj);
+      f[i] = f[i] - om * (f[i] - ei) + pref * si;
+      f[j] = f[j] - om * (f[j] - ej) + pref * sj;
     }
   } else {
     // TRT on the pairs (i, ibar): the symmetric parts are shared, the
-    // antisymmetric parts change sign (same roundings as a per-i loop).
-    // With the model, omega- follows from the adjusted omega+ through the
-    // magic parameter.
+    // antisymmetric parts change sign.  With the model, omega- follows from
+    // the adjusted omega+ through the magic parameter.
     R omp = R(p.omega), omm = R(p.om_m), prp = R(p.pref_p), prm = R(p.pref_m);
     if constexpr (coll_les(COLL)) {
       omp = omega;
@@ -214,29 +265,21 @@ __device__ __forceinline__ R collide(R* f, const KParams& p, bool& unstable) {
       prp = R(1.0) - R(0.5) * omp;
       prm = R(1.0) - R(0.5) * omm;
     }
-    {
-      const R fe = feq_i<Q, R>(0, rho, ux, uy, uz);
-      const R sr = guo_i<Q, R>(0, ux, uy, uz, Fx, Fy, Fz);
-      const R fp = R(0.5) * (f[0] + f[0]), fm = R(0.5) * (f[0] - f[0]);
-      const R ep = R(0.5) * (fe + fe), em = R(0.5) * (fe - fe);
-      const R sp = R(0.5) * (sr + sr), sm = R(0.5) * (sr - sr);
-      f[0] = f[0] - omp * (fp - ep) - omm * (fm - em) + prp * sp + prm * sm;
-    }
+    const R hp = R(0.5) * omp, hm = R(0.5) * omm, gp = R(0.5) * prp, gm = R(0.5) * prm;
+    f[0] = f[0] - omp * (f[0] - fe0) + prp * s0;
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
       const int j = i + 1;
-      const R fei = feq_i<Q, R>(i, rho, ux, uy, uz), fej = feq_i<Q, R>(j, rho, ux, uy, uz);
-      const R si = guo_i<Q, R>(i, ux, uy, uz, Fx, Fy, Fz), sj = guo_i<Q, R>(j, ux, uy, uz, Fx, Fy, Fz);
-      const R fp = R(0.5) * (f[i] + f[j]);
-      const R ep = R(0.5) * (fei + fej);
-      const R sp = R(0.5) * (si + sj);
-      const R fmi = R(0.5) * (f[i] - f[j]), fmj = R(0.5) * (f[j] - f[i]);
-      const R emi = R(0.5) * (fei - fej), emj = R(0.5) * (fej - fei);
-      const R smi = R(0.5) * (si - sj), smj = R(0.5) * (sj - si);
-      const R oi = f[i] - omp * (fp - ep) - omm * (fmi - emi) + prp * sp + prm * smi;
-      const R oj = f[j] - omp * (fp - ep) - omm * (fmj - emj) + prp * sp + prm * smj;
-      f[i] = oi;
-      f[j] = oj;
+      const R cu = cdot<R>(i, ux, uy, uz), cF = cdot<R>(i, Fx, Fy, Fz);
+      R ei, ej, si, sj;
+      feq_pair<R>(W<Q, R>(i) * rho, cu, b, ei, ej);
+      guo_pair<R>(W<Q, R>(i), cu, cF, uF, si, sj);
+      const R A = hp * ((f[i] + f[j]) - (ei + ej));
+      const R B = hm * ((f[i] - f[j]) - (ei - ej));
+      const R C = gp * (si + sj);
+      const R D = gm * (si - sj);
+      f[i] = f[i] - A - B + C + D;
+      f[j] = f[j] - A + B + C - D;
     }
   }
   return rho;
@@ -246,9 +289,39 @@ __device__ __forceinline__ R collide(R* f, const KParams& p, bool& unstable) {
 // - 1.5 u.u)) with drho = rho - 1 (Eq. nm-lbm-equilibrium).
 template <int Q, class R>
 __device__ __forceinline__ R feq_dev(int i, R drho, R rho, R ux, R uy, R uz) {
-  const R cu = R(CX(i)) * ux + R(CY(i)) * uy + R(CZ(i)) * uz;
+  const R cu = cdot<R>(i, ux, uy, uz);
   const R usq = ux * ux + uy * uy + uz * uz;
   return W<Q, R>(i) * (drho + rho * (R(3.0) * cu + R(4.5) * cu * cu - R(1.5) * usq));
+}
+
+// f^eq_i + f^eq_ibar of the free-surface condition (Eq.
+// nm-fslbm-boundary-condition) with each term rounded as by feq_i or
+// feq_dev; the same sum serves i and ibar.  In the deviation formats rg is
+// rho^G - 1 and the terms are deviations.
+template <int Q, class S>
+__device__ __forceinline__ typename S::Real feq_sum(int i, typename S::Real rg, typename S::Real ux,
+                                                    typename S::Real uy, typename S::Real uz,
+                                                    typename S::Real usq) {
+  using R = typename S::Real;
+  const R b = R(1.5) * usq;
+  if constexpr (S::kDev) {
+    const R rgf = R(1.0) + rg, w = W<Q, R>(i);
+    if (i == 0) {
+      const R e = w * (rg + rgf * (R(0.0) - b));
+      return e + e;
+    }
+    const R cu = cdot<R>(i, ux, uy, uz), c3 = R(3.0) * cu, a = R(4.5) * cu * cu;
+    return w * (rg + rgf * (c3 + a - b)) + w * (rg + rgf * (a - c3 - b));
+  } else {
+    const R wr = W<Q, R>(i) * rg;
+    if (i == 0) {
+      const R e = wr * (R(1.0) - b);
+      return e + e;
+    }
+    R ei, ej;
+    feq_pair<R>(wr, cdot<R>(i, ux, uy, uz), b, ei, ej);
+    return ei + ej;
+  }
 }
 
 // Collision of the FP32 engines on deviations d_i = f_i - w_i (the same
@@ -290,7 +363,7 @@ __device__ __forceinline__ float collide_dev(float* d, const KParams& p, bool& u
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
       const float cx = float(CX(i)), cy = float(CY(i)), cz = float(CZ(i));
-      const float cu = cx * ux + cy * uy + cz * uz;
+      const float cu = cdot<float>(i, ux, uy, uz);
       const float es = W<Q, float>(i) * __fmaf_rn(r45 * cu, cu, base);
       const float dn = __fmaf_rn(-2.0f, es, d[i] + d[i + 1]);
       qxx += cx * cx * dn;
@@ -320,8 +393,8 @@ __device__ __forceinline__ float collide_dev(float* d, const KParams& p, bool& u
   for (int i = 1; i < Q; i += 2) {
     const int j = i + 1;
     const float w = W<Q, float>(i);
-    const float cu = float(CX(i)) * ux + float(CY(i)) * uy + float(CZ(i)) * uz;
-    const float cF = float(CX(i)) * Fx + float(CY(i)) * Fy + float(CZ(i)) * Fz;
+    const float cu = cdot<float>(i, ux, uy, uz);
+    const float cF = cdot<float>(i, Fx, Fy, Fz);
     const float es = w * __fmaf_rn(r45 * cu, cu, base);
     const float ea = (3.0f * w) * rho * cu;
     const float ss = w * __fmaf_rn(9.0f * cu, cF, -uF3);

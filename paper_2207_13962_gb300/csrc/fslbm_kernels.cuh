@@ -958,20 +958,18 @@ __device__ __forceinline__ void interface_cell(const DPtrs& d, const KParams& p,
     if (v == 4) v = (__popc(miss) >= 3) ? 3 : p.om3_fb;
     const R rg = rhog[c];  // rho^G (FP64 engine) or rho^G - 1
     const R tie = R(kTie);
+    const R usq = ux * ux + uy * uy + uz * uz;
+    if (v == 1) f[0] = feq_sum<Q, S>(0, rg, ux, uy, uz, usq) - fx[0];  // n^.c_0 = 0: a tie
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      bool rec = (miss >> i) & 1u;
-      const R dot = R(CX(i)) * n0 + R(CY(i)) * n1 + R(CZ(i)) * n2;
-      if (v == 1 && dot >= -tie) rec = true;
-      if (v == 2 && dot > tie) rec = true;
-      if (rec) {
-        const int j = OPP(i);
-        if constexpr (S::kDev) {
-          const R rgf = R(1.0) + rg;
-          f[i] = (feq_dev<Q, R>(i, rg, rgf, ux, uy, uz) + feq_dev<Q, R>(j, rg, rgf, ux, uy, uz)) - fx[j];
-        } else {
-          f[i] = (feq_i<Q, R>(i, rg, ux, uy, uz) + feq_i<Q, R>(j, rg, ux, uy, uz)) - fx[j];
-        }
+    for (int i = 1; i < Q; i += 2) {
+      const int j = i + 1;
+      const R dot = cdot<R>(i, n0, n1, n2);  // -dot for j
+      const bool ri = ((miss >> i) & 1u) || (v == 1 && dot >= -tie) || (v == 2 && dot > tie);
+      const bool rj = ((miss >> j) & 1u) || (v == 1 && dot <= tie) || (v == 2 && dot < -tie);
+      if (ri || rj) {
+        const R e = feq_sum<Q, S>(i, rg, ux, uy, uz, usq);
+        if (ri) f[i] = e - fx[j];
+        if (rj) f[j] = e - fx[i];
       }
     }
     long long s_in = 0;  // the mass-conserving formats: the received values in grid steps
