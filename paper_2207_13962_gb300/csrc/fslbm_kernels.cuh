@@ -1758,7 +1758,7 @@ __global__ void __launch_bounds__(kGeoBlock, kGeoMinBlocks) kb_geometry(const Do
 // of the plan (n + 1 entries each), cleared by kb_plan_front every step.
 __device__ __forceinline__ int* batch_bulk_ctr(const BatchPlan& pl) { return pl.all + pl.n + 1; }
 
-// Units of all domains handed out as in k_bulk, kBulkChunk at a time.
+// Units of all domains handed out as in k_bulk.
 template <int Q, class S, int COLL>
 __device__ __forceinline__ void batch_bulk_sweep(const DomRec* __restrict__ recs, const BatchPlan& pl) {
   const int total = pl.bulk[pl.n];
@@ -1767,19 +1767,7 @@ __device__ __forceinline__ void batch_bulk_sweep(const DomRec* __restrict__ recs
     const DomRec& r = recs[k];
     bulk_unit<Q, S, COLL>(r.d, r.p, r.parity, w - pl.bulk[k], r.d.counts[5]);
   };
-  if constexpr (kBulkChunk > 0) {
-    for (;;) {
-      int base = 0;
-      if ((threadIdx.x & 31) == 0) base = atomicAdd(batch_bulk_ctr(pl), kBulkChunk);
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (base >= total) break;
-      const int end = base + kBulkChunk < total ? base + kBulkChunk : total;
-      for (int w = base; w < end; ++w) unit(w);
-    }
-  } else {
-    const int warps = (gridDim.x * kBulkBlock) >> 5;
-    for (int w = (blockIdx.x * kBulkBlock + threadIdx.x) >> 5; w < total; w += warps) unit(w);
-  }
+  hand_out_units<S>(total, batch_bulk_ctr(pl), unit);
 }
 
 template <int Q, class S, int COLL>
