@@ -262,7 +262,7 @@ fslbm_status fslbm_create(const fslbm_domain* domain, fslbm_lattice lattice,
   ALLOC(d.share, N * sizeof(double));
   ALLOC(d.band[0], N * sizeof(int));
   ALLOC(d.band[1], N * sizeof(int));
-  ALLOC(d.counts, 8 * sizeof(int));
+  ALLOC(d.counts, kCounts * sizeof(int));
   const long long ntiles = (long long)((domain->nx + 7) / 8) * ((domain->ny + 7) / 8) * ((domain->nz + 7) / 8);
   ALLOC(d.tiles[0], ntiles * sizeof(int));
   ALLOC(d.tiles[1], ntiles * sizeof(int));
@@ -546,7 +546,7 @@ fslbm_status fslbm_init(fslbm_ctx* c, const double* fill, const uint8_t* flags,
     c->ops.init_cells(d, c->kp, raw, dfill, dvel, dden, st);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemsetAsync(d.counts, 0, 8 * sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d.counts, 0, kCounts * sizeof(int), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(d.err, 0, 4 * sizeof(int), st);
   // a context initialised again still holds the tile marks of its last step
   if (e == cudaSuccess) {
@@ -1008,7 +1008,7 @@ fslbm_status fslbm_load(fslbm_ctx* c, const void* buf, size_t size) {
   h2d(c->d.Vcur, nb * sizeof(double));
   h2d(c->d.gas_cnt, nb * sizeof(long long));
   if (e == cudaSuccess && nb) e = cudaMemset(c->d.iface_fix, 0, nb * sizeof(long long));
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->d.counts, 0, 8 * sizeof(int), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d.counts, 0, kCounts * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d.err, 0, 4 * sizeof(int), c->stream);
   if (e == cudaSuccess) {
     const size_t nt = (size_t)((c->kp.nx + 7) / 8) * ((c->kp.ny + 7) / 8) * ((c->kp.nz + 7) / 8);

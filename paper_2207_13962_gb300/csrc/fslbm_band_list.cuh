@@ -16,8 +16,7 @@ namespace fslbm {
 // result (the band kernels read time-t neighbours and gather), but
 // neighbouring entries then hold neighbouring cells, so the loads of a warp
 // in the band kernels share sectors.  Appending the surviving cells warp by
-// warp (the batched finalize does, before kb_compact_band rewrites its
-// lists) interleaves runs from unrelated places a little more every step:
+// warp instead interleaves runs from unrelated places a little more every step:
 // on the 160x160x1024 Taylor bubble the interface kernel took 47.8 us just
 // after init and 81 us fifty steps later, 47 us with the list in cell order.
 constexpr int kCompactCells = 16;                       // cells a lane scans
@@ -82,25 +81,16 @@ static __global__ void __launch_bounds__(kBlock) k_compact_band(DPtrs d, KParams
 }
 
 // All domains of a batch, at the end of a batched step (after the buffer
-// swap, so a domain's next list is band[parity]).  The batched finalize has
-// already appended the same cells in warp order and set the list's count;
-// this rewrites the entries in cell order, counting with cnt[k] (n entries,
-// zero before the launch).  chunk_off[k]: prefix of the domains' chunk
-// counts (n + 1 entries).
+// swap, so a domain's next list is band[parity]).  chunk_off[k]: prefix of
+// the domains' chunk counts (n + 1 entries).
 static __global__ void __launch_bounds__(kBlock) kb_compact_band(const DomRec* __restrict__ recs,
-                                                                 const int* __restrict__ chunk_off, int n,
-                                                                 int* cnt) {
+                                                                 const int* __restrict__ chunk_off, int n) {
   const int total = chunk_off[n];
   for (int g = blockIdx.x; g < total; g += gridDim.x) {
-    int lo = 0, hi = n - 1;  // the domain k with chunk_off[k] <= g < chunk_off[k + 1]
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (chunk_off[mid] <= g) lo = mid;
-      else hi = mid - 1;
-    }
-    const DomRec& r = recs[lo];
-    compact_chunk(r.d.flags, r.p.N, (long long)(g - chunk_off[lo]) * kCompactChunk, r.d.band[r.parity],
-                  &cnt[lo]);
+    const int k = find_domain(chunk_off, n, g);
+    const DomRec& r = recs[k];
+    compact_chunk(r.d.flags, r.p.N, (long long)(g - chunk_off[k]) * kCompactChunk, r.d.band[r.parity],
+                  &r.d.counts[r.parity]);
   }
 }
 

@@ -64,6 +64,19 @@ __device__ __forceinline__ int warp_append(int* counter, bool pred) {
   return pred ? base + __popc(b & ((1u << lane) - 1u)) : -1;
 }
 
+// Largest domain k < n with off[k] <= g (off non-decreasing, off[0] = 0).
+__device__ __forceinline__ int find_domain(const int* __restrict__ off, int n, int g) {
+  int lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (off[mid] <= g) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+__device__ __forceinline__ int round32(int v) { return (v + 31) & ~31; }
+
 // Block-wide exclusive prefix sum (one block) of values f(k), k < n, into
 // off[0..n]; f must not read off.
 template <class F>
@@ -436,6 +449,19 @@ __device__ __forceinline__ typename S::T store_w(typename S::Real v, int i) {
     return S::stored(v);
   else
     return S::store(v, W<Q, typename S::Real>(i));
+}
+
+// Weight of a direction with |c|^2 = n2 (W as a function of a run-time
+// value), and the stored value of a working one in such a direction.
+template <int Q, class R>
+__device__ __forceinline__ R lane_weight(int n2) {
+  if constexpr (Q == 19) return n2 == 0 ? R(1.0 / 3.0) : n2 == 1 ? R(1.0 / 18.0) : R(1.0 / 36.0);
+  else return n2 == 0 ? R(8.0 / 27.0) : n2 == 1 ? R(2.0 / 27.0) : n2 == 2 ? R(1.0 / 54.0) : R(1.0 / 216.0);
+}
+template <class S>
+__device__ __forceinline__ typename S::T lane_store(typename S::Real v, typename S::Real w) {
+  if constexpr (S::kDev) return S::stored(v);
+  else return S::store(v, w);
 }
 
 // ------------------------------------------- mass-conserving formats

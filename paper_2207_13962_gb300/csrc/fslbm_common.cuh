@@ -383,13 +383,15 @@ struct DPtrs {
   uint8_t* conv;
   uint8_t* cfin;
   uint8_t* claim;
-  uint8_t* rcv;    // 1: an interface cell next to a cell that converts this
-                   // step (set by the count kernel, cleared by apply)
+  uint8_t* rcv;    // 1: an interface cell on the receiver list (next to a
+                   // cell that converts; set by the count kernel, cleared
+                   // by apply)
   double* share;
   int* band[2];
   int* counts;   // [0],[1]: band list counts; [2]: new-cell list count;
                  // [3],[4]: geometry tile list counts; [5]: segment count;
-                 // [6], [7]: the step's bulk-unit and tile hand-out
+                 // [6], [7]: the step's bulk-unit and tile hand-out;
+                 // [8], [9]: converting cells and excess receivers
   int* tiles[2]; // geometry tiles (8^3) holding interface cells
   int* tile_mark;
   int* segs;     // 32-cell segments (linear index / 32) holding liquid;
@@ -402,7 +404,7 @@ struct DPtrs {
                     // same arithmetic as post_moments, read for new cells
   double* m_next;
   double* phi_next;
-  double* rho_band;
+  double* rho_band;  // FP64: rho of the band cells' collision, by cell
   double* V0;
   double* pV;
   double* Vcur;
@@ -426,13 +428,14 @@ struct DomRec {
 // the units of each batched kernel, recomputed on the device every step:
 //   tiles: geometry tiles; bulk: warp units of the bulk sweep;
 //   band: interface cells rounded up to a multiple of 32 (warp-aligned);
-//   all: interface + new interface cells rounded up to a multiple of 32.
+// ctr: the hand-out counters of the bulk sweep and of the fused tiles.
 struct BatchPlan {
   int n;
   int* tiles;
   int* bulk;
   int* band;
-  int* all;
+  int* ctr;
 };
+constexpr int kCounts = 16;  // ints of DPtrs::counts
 
 }  // namespace fslbm

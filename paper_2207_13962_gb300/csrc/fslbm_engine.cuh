@@ -8,7 +8,6 @@
 
 #include "fslbm_kernels.cuh"
 #include "fslbm_band_list.cuh"
-#include "fslbm_apply.cuh"
 
 namespace fslbm {
 
@@ -93,10 +92,9 @@ struct Engine {
         k_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(d, p, parity);
       });
       if (ev) ev->mark(3, st);
-      // three resident blocks per SM (75 registers): about one band cell a thread
-      k_resolve<Q><<<band_grid * 3 / 2, kBlock, 0, st>>>(d, p, parity);
+      k_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
       if (ev) ev->mark(4, st);
-      k_count<Q><<<band_grid, kBlock, 0, st>>>(d, p, parity);
+      k_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
       if (ev) ev->mark(5, st);
       // the two independent parts of the apply stage, side by side in the
       // graph (one after the other while stages are timed)
@@ -105,9 +103,9 @@ struct Engine {
         cudaEventRecord(fk->fork, st);
         cudaStreamWaitEvent(fk->side, fk->fork, 0);
       }
-      k_apply_new<Q, S><<<band_grid, 128, 0, side ? fk->side : st>>>(d, p, parity);
+      k_apply<Q, S, true, false><<<band_grid * 2, kBlock, 0, side ? fk->side : st>>>(d, p, parity);
       if (side) cudaEventRecord(fk->join, fk->side);
-      k_apply_band<Q, S><<<band_grid * 2, 128, 0, st>>>(d, p, parity);
+      k_apply<Q, S, false, true><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
       if (side) cudaStreamWaitEvent(st, fk->join, 0);
       if (ev) ev->mark(6, st);
       k_finalize<<<band_grid, kBlock, 0, st>>>(d, p, parity);
@@ -156,12 +154,12 @@ struct Engine {
       k_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(d, p, parity);
     });
     if (ev) ev->mark(3, st);
-    k_resolve<Q><<<band_grid, kBlock, 0, st>>>(d, p, parity);
+    k_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
     if (ev) ev->mark(4, st);
-    k_count<Q><<<band_grid, kBlock, 0, st>>>(d, p, parity);
+    k_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
     if (ev) ev->mark(5, st);
     if (forked) cudaStreamWaitEvent(st, fk->join, 0);
-    k_apply<Q, S><<<band_grid * 2, 128, 0, st>>>(d, p, parity);
+    k_apply<Q, S, true, true><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
     if (ev) ev->mark(6, st);
     k_finalize<<<band_grid, kBlock, 0, st>>>(d, p, parity);
     k_compact_band<<<compact_grid(p, band_grid), kBlock, 0, st>>>(d, p, parity);
@@ -186,10 +184,9 @@ struct Engine {
       with_coll(collision, [&](auto C) {
         kb_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(recs, pl);
       });
-      kb_resolve<Q><<<band_grid, kBlock, 0, st>>>(recs, pl);
-      kb_count<Q><<<band_grid, kBlock, 0, st>>>(recs, pl);
-      kb_plan_back<<<1, 1024, 0, st>>>(recs, pl);
-      kb_apply<Q, S><<<band_grid * 2, 128, 0, st>>>(recs, pl);
+      kb_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
+      kb_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
+      kb_apply<Q, S, true, true><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
       kb_finalize<<<band_grid, kBlock, 0, st>>>(recs, pl);
       kb_bubble_end<<<pl.n, 256, 0, st>>>(recs);
       (void)fk;
@@ -205,11 +202,16 @@ struct Engine {
     with_coll(collision, [&](auto C) {
       kb_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(recs, pl);
     });
-    kb_resolve<Q><<<band_grid, kBlock, 0, st>>>(recs, pl);
-    kb_count<Q><<<band_grid, kBlock, 0, st>>>(recs, pl);
-    kb_plan_back<<<1, 1024, 0, st>>>(recs, pl);
+    kb_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
+    kb_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
     cudaStreamWaitEvent(st, fk->join, 0);
-    kb_apply<Q, S><<<band_grid * 2, 128, 0, st>>>(recs, pl);
+    // the new cells' FP64 chains beside the receivers'
+    cudaEventRecord(fk->fork, st);
+    cudaStreamWaitEvent(fk->side, fk->fork, 0);
+    kb_apply<Q, S, true, false><<<band_grid * 2, kBlock, 0, fk->side>>>(recs, pl);
+    cudaEventRecord(fk->join, fk->side);
+    kb_apply<Q, S, false, true><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
+    cudaStreamWaitEvent(st, fk->join, 0);
     kb_finalize<<<band_grid, kBlock, 0, st>>>(recs, pl);
     kb_bubble_end<<<pl.n, 256, 0, st>>>(recs);
   }
@@ -274,13 +276,15 @@ struct Engine {
       o.bulk_fn[7] = (const void*)&k_bulk<Q, S, 7>;
     }
     o.bulk_blocks_per_sm = bulk_blocks_per_sm();
-    o.step_launches = 8;  // fused: the apply stage is two kernels
+    // bulk and geometry (one launch when fused), interface, resolve, count,
+    // apply (two launches when fused), finalize, list rebuild
+    o.step_launches = 8;
     o.bulk_smem = kTmaBulk ? tma_smem<Q, typename S::T>() : kFusedGeo ? geometry_smem<typename S::Real>() : 0;
     o.batch_step = &batch_step;
-    // two plan kernels, geometry, bulk sweep, interface update, resolve,
-    // count, apply, finalize, bubbles + buffer swap (one less when the
-    // geometry is folded into the sweep)
-    o.batch_step_launches = kFusedGeo ? 10 : 11;  // with kb_compact_band, launched by the batch
+    // plan, geometry, bulk sweep (one launch when fused), interface update,
+    // resolve, count, apply (two in FP64), finalize, bubbles + buffer swap,
+    // and kb_compact_band, launched by the batch
+    o.batch_step_launches = kFusedGeo ? 9 : 11;
     if constexpr (kFusedGeo) {
       const void* fns[8] = {(const void*)&kb_bulk_geo<Q, S, 0>, (const void*)&kb_bulk_geo<Q, S, 1>,
                             (const void*)&kb_bulk_geo<Q, S, 2>, (const void*)&kb_bulk_geo<Q, S, 3>,

@@ -7,10 +7,12 @@
 //   k_bulk       grid   pull stream + bounce-back + collide of liquid cells
 //   k_interface  band   pull, free-surface BC of the chosen variant, mass
 //                       exchange, fill update, collide, conversion marks
-//   k_resolve    band   conflict rule, claims of gas/liquid neighbours
-//   k_count      band   excess-mass receivers, deferral, shares
-//   k_apply      band+new  excess gather, new interface cells' PDFs
-//   k_finalize   band+new  final flags, next interface list, bubble sums
+//   k_resolve    list+band  conflict rule, claims of gas/liquid neighbours;
+//                       commit of m and phi
+//   k_count      list   excess-mass receivers, deferral, shares
+//   k_apply      lists  excess gather, new interface cells' PDFs
+//   k_finalize   band+new  final flags, tile and segment marks, bubble sums
+//   k_compact_band grid the next interface list
 //   k_bubble     1 block   bubble volume pressure
 // The interface work runs only on the compacted list of interface cells
 // ("band") and on the cells that conversion turns into interface cells.
@@ -23,6 +25,7 @@
 #pragma once
 
 #include "fslbm_bulk_tma.cuh"
+#include "fslbm_convert.cuh"
 #include <type_traits>
 
 namespace fslbm {
@@ -740,11 +743,13 @@ __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, 
   }
 
 // Resets the work-list counters that this step fills (next band list, new
-// cells, next tile list).
+// cells, next tile list, converting cells, receivers).
 __device__ __forceinline__ void reset_step_counts(const DPtrs& d, int parity) {
   d.counts[parity ^ 1] = 0;
   d.counts[2] = 0;
   d.counts[3 + (parity ^ 1)] = 0;
+  *conv_count(d) = 0;
+  *recv_count(d) = 0;
 }
 
 template <int Q, class S>
@@ -1050,8 +1055,10 @@ __device__ __forceinline__ void interface_cell(const DPtrs& d, const KParams& p,
     }
     d.m_next[k] = mn;
     d.phi_next[k] = phin;
-    d.rho_band[k] = rho;
-    d.mark[c] = (phin > 1.0 + p.eps) ? CV_TOL : (phin < -p.eps) ? CV_TOG : CV_NONE;
+    if constexpr (!S::kDev) d.rho_band[c] = rho;
+    const uint8_t mark = (phin > 1.0 + p.eps) ? CV_TOL : (phin < -p.eps) ? CV_TOG : CV_NONE;
+    d.mark[c] = mark;
+    if (mark != CV_NONE) append_conversion(d, parity, c);
   }
 
 template <int Q, class S, int COLL>
@@ -1063,357 +1070,7 @@ __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) k_interfac
   if (bad) d.err[0] = 1;
 }
 
-// -------------------------------------------------------------- conversion
-// These passes are chains of dependent neighbour reads over a few hundred
-// converting cells, so their duration is the number of round trips to
-// memory along the longest chain.  Each pass reads the neighbours' values
-// one level at a time for all directions together (types, then the values
-// the types select, then the values those select) and writes only after
-// the last read; the arithmetic and its order are those of a per-direction
-// loop.
-
-// Neighbour indices of (x, y, z) and their types (T_OBST outside the domain).
-template <int Q>
-__device__ __forceinline__ void neighbour_types(const DPtrs& d, const KParams& p, int x, int y,
-                                                int z, int* nid, uint8_t* nt) {
-#pragma unroll
-  for (int i = 1; i < Q; ++i) nid[i] = nbr(p, x, y, z, CX(i), CY(i), CZ(i));
-#pragma unroll
-  for (int i = 1; i < Q; ++i) nt[i] = nid[i] >= 0 ? (uint8_t)(d.flags[nid[i]] & F_TYPE) : (uint8_t)T_OBST;
-}
-
-// Commit m, phi; conflict rule (a cell marked for gas stays interface next
-// to a cell marked for liquid); claim gas neighbours of cells turning liquid
-// and liquid neighbours of cells turning gas as new interface cells.
-template <int Q>
-__device__ __forceinline__ void resolve_cell(const DPtrs& d, const KParams& p, int parity, int k) {
-  const int c = d.band[parity][k];
-  uint8_t cv = d.mark[c];
-  d.mass[c] = d.m_next[k];
-  d.phi[c] = d.phi_next[k];
-  if (cv == CV_NONE) {
-    d.conv[c] = CV_NONE;
-    return;
-  }
-  int x, y, z;
-  decode(p, c, x, y, z);
-  int nid[Q];
-  uint8_t nt[Q];
-  neighbour_types<Q>(d, p, x, y, z, nid, nt);
-  if (cv == CV_TOG) {
-    uint8_t mk[Q];
-#pragma unroll
-    for (int i = 1; i < Q; ++i) mk[i] = nt[i] == T_IFACE ? d.mark[nid[i]] : (uint8_t)CV_NONE;
-#pragma unroll
-    for (int i = 1; i < Q; ++i)
-      if (mk[i] == CV_TOL) cv = CV_NONE;
-  }
-  d.conv[c] = cv;
-  if (cv == CV_NONE) return;
-  const int want = (cv == CV_TOL) ? T_GAS : T_LIQ;
-  // claim first (the atomics are independent of one another), then reserve
-  // all of this cell's new entries with one atomic (the list's order enters
-  // no result)
-  unsigned fresh = 0u;
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    if (nt[i] != want) continue;
-    const int nb = nid[i];
-    unsigned* word = (unsigned*)(d.claim + (nb & ~3));
-    const unsigned bit = 1u << (8 * (nb & 3));
-    const unsigned old = atomicOr(word, bit);
-    if (!(old & bit)) fresh |= 1u << i;
-  }
-  if (!fresh) return;
-  int pos = atomicAdd(&d.counts[2], __popc(fresh));
-#pragma unroll
-  for (int i = 1; i < Q; ++i)
-    if ((fresh >> i) & 1u) d.newlist[pos++] = nid[i];
-}
-
-template <int Q>
-__global__ void __launch_bounds__(kBlock) k_resolve(DPtrs d, KParams p, int parity) {
-  const int n = d.counts[parity];
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-    resolve_cell<Q>(d, p, parity, k);
-}
-
-// Excess-mass receivers (Eq. nm-fslbm-excess-mass): interface cells after
-// conversion in the lattice neighbourhood (interface cells that do not
-// convert, and the gas or liquid cells that conversion claims); none -> the
-// conversion is deferred.
-template <int Q>
-__device__ __forceinline__ void count_cell(const DPtrs& d, const KParams& p, int parity, int k) {
-  const int c = d.band[parity][k];
-  const uint8_t cv = d.conv[c];
-  if (cv == CV_NONE) {
-    d.cfin[c] = CV_NONE;
-    return;
-  }
-  const double m = d.mass[c];
-  const double rb = d.rho_band[k];
-  int x, y, z;
-  decode(p, c, x, y, z);
-  int nid[Q];
-  uint8_t nt[Q];
-  neighbour_types<Q>(d, p, x, y, z, nid, nt);
-  uint8_t nv[Q];  // conv of interface neighbours, claim of gas and liquid ones
-#pragma unroll
-  for (int i = 1; i < Q; ++i)
-    nv[i] = nt[i] == T_IFACE ? d.conv[nid[i]] : nt[i] != T_OBST ? d.claim[nid[i]] : (uint8_t)0;
-  int nrecv = 0;
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const bool post = nt[i] == T_IFACE ? nv[i] == CV_NONE : nt[i] != T_OBST && nv[i] != 0;
-    nrecv += post ? 1 : 0;
-  }
-  if (nrecv == 0) {
-    d.cfin[c] = CV_DEFER;
-    return;
-  }
-  const double mex = (cv == CV_TOL) ? (m - rb) : m;
-  d.share[c] = mex / (double)nrecv;
-  d.cfin[c] = cv;
-  // flag the interface neighbours, which gather this cell's share: the
-  // others skip the gather (it would add nothing)
-#pragma unroll
-  for (int i = 1; i < Q; ++i)
-    if (nt[i] == T_IFACE) d.rcv[nid[i]] = 1;
-}
-
-template <int Q>
-__global__ void __launch_bounds__(kBlock) k_count(DPtrs d, KParams p, int parity) {
-  const int n = d.counts[parity];
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
-    count_cell<Q>(d, p, parity, k);
-}
-
-__device__ __forceinline__ bool is_converted(uint8_t f) { return f == CV_TOL || f == CV_TOG; }
-
-// 2-bit fields per direction (types T_*, conversion states CV_*)
-__device__ __forceinline__ int field2(uint64_t m, int i) { return (int)((m >> (2 * i)) & 3u); }
-
-// Sum of the excess shares of converted neighbours, in direction order.
-// cfm: 2-bit cfin of the interface neighbours (CV_NONE elsewhere).
-template <int Q>
-__device__ __forceinline__ double gather_shares(const DPtrs& d, const int* nid, uint64_t cfm) {
-  double sh[Q];
-#pragma unroll
-  for (int i = 1; i < Q; ++i) sh[i] = is_converted((uint8_t)field2(cfm, i)) ? d.share[nid[i]] : 0.0;
-  double s = 0.0;
-#pragma unroll
-  for (int i = 1; i < Q; ++i)
-    if (is_converted((uint8_t)field2(cfm, i))) s = s + sh[i];
-  return s;
-}
-
-// Excess gather for all interface cells after conversion; PDFs of new
-// interface cells from gas: f* = f^eq(mean rho, mean u) over liquid and old
-// interface neighbours; new interface cells from liquid: m = rho, phi = 1.
-template <int Q, class S>
-__device__ __forceinline__ void apply_cell(const DPtrs& d, const KParams& p, int parity, int k) {
-  using R = typename S::Real;
-  using T = typename S::T;
-  // the new cells come first: their dependent chains are the longest, so
-  // they start with the launch
-  const int nnew = d.counts[2];
-  T* __restrict__ B = (T*)d.pdf[parity ^ 1];
-  const long long Np = p.Np;
-
-  const bool is_band = k >= nnew;
-  if (is_band) k -= nnew;
-  const int c = is_band ? d.band[parity][k] : d.newlist[k];
-  int x, y, z;
-  int nid[Q];
-  if (is_band) {
-    const bool gather = d.rcv[c] != 0;
-    const uint8_t f = d.cfin[c];
-    if (gather) d.rcv[c] = 0;
-    if (f == CV_TOL) {
-      d.phi[c] = 1.0;
-      d.mass[c] = d.rho_band[k];
-      return;
-    }
-    if (f == CV_TOG) {
-      d.phi[c] = 0.0;
-      d.mass[c] = 0.0;
-      return;
-    }
-    // a deferred cell stays interface and keeps its mass: it was not counted
-    // among its converting neighbours' receivers
-    if (f == CV_DEFER) return;
-    const double m0 = d.mass[c];
-    // an interface cell that no converted cell flagged receives nothing:
-    // m + 0 and (m + 0) / rho are the m and phi that k_resolve stored
-    // (m_next and phi_next = m_next / rho), unless m is -0
-    if (!gather && !(m0 == 0.0 && signbit(m0))) return;
-    const double rb = d.rho_band[k];
-    double s = 0.0;
-    if (gather) {
-      decode(p, c, x, y, z);
-#pragma unroll
-      for (int i = 1; i < Q; ++i) nid[i] = nbr(p, x, y, z, CX(i), CY(i), CZ(i));
-      unsigned ifm = 0u;  // interface neighbours
-#pragma unroll
-      for (int i = 1; i < Q; ++i)
-        if (nid[i] >= 0 && (d.flags[nid[i]] & F_TYPE) == T_IFACE) ifm |= 1u << i;
-      uint64_t cfm = 0;
-#pragma unroll
-      for (int i = 1; i < Q; ++i)
-        if ((ifm >> i) & 1u) cfm |= (uint64_t)(d.cfin[nid[i]] & 3u) << (2 * i);
-      s = gather_shares<Q>(d, nid, cfm);
-    }
-    const double m = m0 + s;
-    d.mass[c] = m;
-    d.phi[c] = m / rb;
-    return;
-  }
-
-  // a new interface cell (gas or liquid before this step)
-  const uint8_t fl = d.flags[c];
-  const int t = fl & F_TYPE;
-  decode(p, c, x, y, z);
-#pragma unroll
-  for (int i = 1; i < Q; ++i) nid[i] = nbr(p, x, y, z, CX(i), CY(i), CZ(i));
-  uint64_t ntm = 0;
-#pragma unroll
-  for (int i = 1; i < Q; ++i)
-    ntm |= (uint64_t)(nid[i] >= 0 ? (d.flags[nid[i]] & F_TYPE) : T_OBST) << (2 * i);
-  uint64_t cfm = 0;   // cfin of interface neighbours
-  uint32_t clm = 0u;  // claimed gas or liquid neighbours
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const int nt = field2(ntm, i);
-    if (nt == T_IFACE) cfm |= (uint64_t)(d.cfin[nid[i]] & 3u) << (2 * i);
-    if ((nt == T_GAS || nt == T_LIQ) && d.claim[nid[i]] != 0) clm |= 1u << i;
-  }
-  const double s = gather_shares<Q>(d, nid, cfm);
-  if (t == T_GAS) {
-    // neighbours that stay or turn liquid, or stay interface
-    unsigned use = 0u;
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const int nt = field2(ntm, i);
-      if (nt == T_IFACE && field2(cfm, i) != CV_TOG) use |= 1u << i;
-      if (nt == T_LIQ && !((clm >> i) & 1u)) use |= 1u << i;
-    }
-    double sr = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-    int cnt = 0;
-    unsigned liq_use = 0u;
-#pragma unroll
-    for (int i = 1; i < Q; ++i)
-      if (((use >> i) & 1u) && field2(ntm, i) == T_LIQ) liq_use |= 1u << i;
-    if (liq_use) {
-      // liquid neighbours (none next to a gas cell while the interface layer
-      // is closed) form their moments from the stored PDFs: direction order
-      for (int i = 1; i < Q; ++i) {
-        if (!((use >> i) & 1u)) continue;
-        double rn;
-        R un[3];
-        if (field2(ntm, i) == T_IFACE) {
-          const R* mu = (const R*)d.mom_u;
-          rn = d.mom_rho[nid[i]];
-          un[0] = mu[3LL * nid[i] + 0];
-          un[1] = mu[3LL * nid[i] + 1];
-          un[2] = mu[3LL * nid[i] + 2];
-        } else {
-          post_moments<Q, S>(B, Np, nid[i], p, rn, un);
-        }
-        sr = sr + rn;
-        sx = sx + (double)un[0];
-        sy = sy + (double)un[1];
-        sz = sz + (double)un[2];
-        ++cnt;
-      }
-    }
-    // moments cached by the interface kernel, read a few directions at a time
-    constexpr int kChunk = 5;
-#pragma unroll
-    for (int i0 = 1; liq_use == 0u && i0 < Q; i0 += kChunk) {
-      double rn[kChunk];
-      R un[kChunk][3];
-#pragma unroll
-      for (int a = 0; a < kChunk; ++a) {
-        const int i = i0 + a;
-        if (i < Q && ((use >> i) & 1u) && field2(ntm, i) == T_IFACE) {
-          const R* mu = (const R*)d.mom_u;
-          rn[a] = d.mom_rho[nid[i]];
-          un[a][0] = mu[3LL * nid[i] + 0];
-          un[a][1] = mu[3LL * nid[i] + 1];
-          un[a][2] = mu[3LL * nid[i] + 2];
-        }
-      }
-#pragma unroll
-      for (int a = 0; a < kChunk; ++a) {
-        const int i = i0 + a;
-        if (i >= Q || !((use >> i) & 1u)) continue;
-        sr = sr + rn[a];
-        sx = sx + (double)un[a][0];
-        sy = sy + (double)un[a][1];
-        sz = sz + (double)un[a][2];
-        ++cnt;
-      }
-    }
-    double rb = 1.0, ub0 = 0.0, ub1 = 0.0, ub2 = 0.0;
-    if (cnt > 0) {
-      rb = sr / (double)cnt;
-      ub0 = sx / (double)cnt;
-      ub1 = sy / (double)cnt;
-      ub2 = sz / (double)cnt;
-    }
-    const uint32_t wm = (fl & F_NEAR_WALL) ? d.wallmask[c] : 0u;
-    R fn[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      if constexpr (S::kDev)
-        fn[i] = feq_dev<Q, R>(i, R(rb - 1.0), R(rb), R(ub0), R(ub1), R(ub2));
-      else
-        fn[i] = feq_i<Q, R>(i, R(rb), R(ub0), R(ub1), R(ub2));
-    }
-    bool over = false;
-    const long long s_new = S::kExactRest ? __double2ll_rn((rb - 1.0) * (double)(1LL << grid_shift<S>())) : 0;
-    store_cell<Q, S>(B, Np, c, fn, s_new, over);
-    if (over) d.err[0] = 1;
-    if (fl & F_NEAR_WALL) write_reflected<Q, S>(d, p, B, c, wm, (fl & F_WRAP) != 0, fn);
-    const double m = 0.0 + s;
-    d.mass[c] = m;
-    d.phi[c] = m / rb;
-  } else {  // from liquid
-    int bb[Q];
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const int nt = field2(ntm, i);
-      const bool gas_after = (nt == T_GAS && !((clm >> i) & 1u)) || (nt == T_IFACE && field2(cfm, i) == CV_TOG);
-      bb[i] = gas_after ? d.bid[nid[i]] : -1;
-    }
-    double rn;
-    R un[3];
-    post_moments<Q, S>(B, Np, c, p, rn, un);
-    int best = -1;
-#pragma unroll
-    for (int i = 1; i < Q; ++i)
-      if (bb[i] >= 0 && (best < 0 || bb[i] < best)) best = bb[i];
-    const double m = rn + s;
-    d.mass[c] = m;
-    d.phi[c] = m / rn;
-    d.bid[c] = best;
-  }
-}
-
-template <int Q, class S>
-__global__ void __launch_bounds__(128) k_apply(DPtrs d, KParams p, int parity) {
-  // the new interface cells (long dependent chains) are dealt round-robin
-  // over the blocks, cell j to thread j / G of block j mod G, so that they
-  // spread over all SMs instead of filling the first blocks; the band cells
-  // follow in order
-  const int nnew = d.counts[2];
-  const int total = gridDim.x * blockDim.x;
-  for (int j = threadIdx.x * gridDim.x + blockIdx.x; j < nnew; j += total) apply_cell<Q, S>(d, p, parity, j);
-  const int nband = d.counts[parity];
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nband; k += total)
-    apply_cell<Q, S>(d, p, parity, nnew + k);
-}
-
+// -------------------------------------------------------------- finalize
 // Fixed-point bubble-volume term round((1 - phi) 2^32).
 __device__ __forceinline__ long long vol_fix(double one_minus_phi) {
   return __double2ll_rn(one_minus_phi * 4294967296.0);
@@ -1472,91 +1129,83 @@ static __global__ void k_tiles_of_band(DPtrs d, KParams p, int parity) {
   }
 }
 
-// Final flags, next interface list, bubble gas counts and interface sums.
-// Entries [base, base + 32) of the band + new-cell list (every lane of the
-// warp calls it).  kAppend: append the cells that stay or become interface
-// to the next interface list (the batched step); a single domain rebuilds
-// that list in cell order with k_compact_band instead.
-template <bool kAppend = true>
-__device__ __forceinline__ void finalize_warp(const DPtrs& d, const KParams& p, int parity,
-                                              int base) {
-  const int* __restrict__ band = d.band[parity];
-  int* __restrict__ next = d.band[parity ^ 1];
-  const int nb_ = d.counts[parity];
-  const int total = nb_ + d.counts[2];
+// Final flags, tile and segment marks, bubble gas counts and interface sums
+// of one cell a lane (c < 0: none), a band cell or a new interface cell;
+// every lane of the warp calls it.  The interface list of the next step is
+// rebuilt from the flags afterwards (compact_chunk).
+__device__ __forceinline__ void finalize_lane(const DPtrs& d, const KParams& p, int parity, int c,
+                                              bool is_band) {
   const int lane = threadIdx.x & 31;
-
-    const int k = base + lane;
-    bool keep = false, to_liq = false;
-    int c = -1, bub = -1, dgas = 0;
-    long long vfix = 0;
-    if (k < total) {
-      const bool is_band = k < nb_;
-      c = is_band ? band[k] : d.newlist[k - nb_];
-      const uint8_t fl = d.flags[c];
-      const int b = d.bid[c];
-      if (is_band) {
-        const uint8_t f = d.cfin[c];
-        if (f == CV_TOL) {
-          d.flags[c] = (fl & ~F_TYPE) | T_LIQ;
-          d.bid[c] = -1;
-          to_liq = true;
-        } else if (f == CV_TOG) {
-          d.flags[c] = (fl & ~F_TYPE) | T_GAS;
-          dgas = 1;
-        } else {
-          keep = true;
-        }
+  bool keep = false, to_liq = false;
+  int bub = -1, dgas = 0;
+  long long vfix = 0;
+  if (c >= 0) {
+    const uint8_t fl = d.flags[c];
+    const int b = d.bid[c];
+    if (is_band) {
+      const uint8_t f = d.cfin[c];
+      if (f != CV_NONE) {  // the marks of a listed cell are spent
+        d.cfin[c] = CV_NONE;
+        d.conv[c] = CV_NONE;
+      }
+      if (f == CV_TOL) {
+        d.flags[c] = (fl & ~F_TYPE) | T_LIQ;
+        d.bid[c] = -1;
+        to_liq = true;
+      } else if (f == CV_TOG) {
+        d.flags[c] = (fl & ~F_TYPE) | T_GAS;
+        dgas = 1;
       } else {
-        if ((fl & F_TYPE) == T_GAS) dgas = -1;
-        d.flags[c] = (fl & ~F_TYPE) | T_IFACE;
-        d.claim[c] = 0;
         keep = true;
       }
-      if (p.bubble_model && b >= 0) {
-        bub = b;
-        if (keep) vfix = vol_fix(1.0 - d.phi[c]);
-      }
-    }
-    if (p.bubble_model) {
-      // integer sums per bubble id present in the warp, one atomic each
-      // (integer addition: the result does not depend on the order)
-      unsigned remaining = 0xffffffffu;
-      while (remaining) {
-        const int leader = __ffs(remaining) - 1;
-        const int bb = __shfl_sync(0xffffffffu, bub, leader);
-        const bool mine = (bub == bb);
-        long long sv = mine ? vfix : 0, sg = mine ? (long long)dgas : 0;
-        for (int o = 16; o > 0; o >>= 1) {
-          sv += __shfl_xor_sync(0xffffffffu, sv, o);
-          sg += __shfl_xor_sync(0xffffffffu, sg, o);
-        }
-        if (lane == leader && bb >= 0) {
-          if (sv) atomicAdd((unsigned long long*)&d.iface_fix[bb], (unsigned long long)sv);
-          if (sg) atomicAdd((unsigned long long*)&d.gas_cnt[bb], (unsigned long long)sg);
-        }
-        remaining &= ~__ballot_sync(0xffffffffu, mine);
-      }
-    }
-    if constexpr (kAppend) {
-      const int pos = warp_append(&d.counts[parity ^ 1], keep);
-      if (keep) next[pos] = c;
     } else {
-      (void)next;
+      if ((fl & F_TYPE) == T_GAS) dgas = -1;
+      d.flags[c] = (fl & ~F_TYPE) | T_IFACE;
+      d.claim[c] = 0;
+      keep = true;
     }
-    mark_tile(d, p, keep ? c : -1, d.tiles[parity ^ 1], &d.counts[3 + (parity ^ 1)]);
-    mark_seg(d, to_liq ? c : -1);
+    if (p.bubble_model && b >= 0) {
+      bub = b;
+      if (keep) vfix = vol_fix(1.0 - d.phi[c]);
+    }
   }
+  if (p.bubble_model) {
+    // integer sums per bubble id present in the warp, one atomic each
+    // (integer addition: the result does not depend on the order)
+    unsigned remaining = __ballot_sync(0xffffffffu, bub >= 0);
+    while (remaining) {
+      const int leader = __ffs(remaining) - 1;
+      const int bb = __shfl_sync(0xffffffffu, bub, leader);
+      const bool mine = (bub == bb);
+      long long sv = mine ? vfix : 0, sg = mine ? (long long)dgas : 0;
+      for (int o = 16; o > 0; o >>= 1) {
+        sv += __shfl_xor_sync(0xffffffffu, sv, o);
+        sg += __shfl_xor_sync(0xffffffffu, sg, o);
+      }
+      if (lane == leader) {
+        if (sv) atomicAdd((unsigned long long*)&d.iface_fix[bb], (unsigned long long)sv);
+        if (sg) atomicAdd((unsigned long long*)&d.gas_cnt[bb], (unsigned long long)sg);
+      }
+      remaining &= ~__ballot_sync(0xffffffffu, mine);
+    }
+  }
+  mark_tile(d, p, keep ? c : -1, d.tiles[parity ^ 1], &d.counts[3 + (parity ^ 1)]);
+  mark_seg(d, to_liq ? c : -1);
+}
 
 static __global__ void __launch_bounds__(kBlock) k_finalize(DPtrs d, KParams p, int parity) {
-  const int total = d.counts[parity] + d.counts[2];
+  const int nband = d.counts[parity], nnew = d.counts[2];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     d.counts[6] = 0;  // the next step's bulk hand-out
     d.counts[7] = 0;  // and geometry-tile hand-out
   }
+  const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  for (int base = wid * 32; base < total; base += warps * 32) finalize_warp<false>(d, p, parity, base);
+  for (int base = wid * 32; base < nband; base += warps * 32)
+    finalize_lane(d, p, parity, base + lane < nband ? d.band[parity][base + lane] : -1, true);
+  for (int base = wid * 32; base < nnew; base += warps * 32)
+    finalize_lane(d, p, parity, base + lane < nnew ? d.newlist[base + lane] : -1, false);
 }
 
 // p^V_b = p^V_b(0) V_b(0) / V_b (Eq. nm-fslbm-pressure-volume).
@@ -1708,39 +1357,19 @@ __global__ void k_to_caller(const T* __restrict__ st, T* __restrict__ ext, KPara
 // so a warp never straddles two domains and the warp-collective code of the
 // single-domain bodies runs unchanged.
 
-// Largest domain k < n with off[k] <= g (off non-decreasing, off[0] = 0).
-__device__ __forceinline__ int find_domain(const int* __restrict__ off, int n, int g) {
-  int lo = 0, hi = n;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (off[mid] <= g) lo = mid;
-    else hi = mid;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ int round32(int v) { return (v + 31) & ~31; }
-
 // Plan of the first phase (before geometry): resets the counters this step
 // fills and lays out tiles, bulk warp units and band cells.
 static __global__ void kb_plan_front(DomRec* recs, BatchPlan pl) {
   constexpr int kGroups = 32 / kSegCells;
   if (threadIdx.x == 0) {
-    *(pl.all + pl.n + 1) = 0;  // the bulk sweep's hand-out counter
-    *(pl.all + pl.n + 2) = 0;  // and the fused sweep's tile counter
+    pl.ctr[0] = 0;  // the bulk sweep's hand-out counter
+    pl.ctr[1] = 0;  // and the fused sweep's tile counter
   }
   for (int k = threadIdx.x; k < pl.n; k += blockDim.x) reset_step_counts(recs[k].d, recs[k].parity);
   __syncthreads();
   block_prefix(pl.n, pl.tiles, [&](int k) { return recs[k].d.counts[3 + recs[k].parity]; });
   block_prefix(pl.n, pl.bulk, [&](int k) { return (recs[k].d.counts[5] + kGroups - 1) / kGroups; });
   block_prefix(pl.n, pl.band, [&](int k) { return round32(recs[k].d.counts[recs[k].parity]); });
-}
-
-// Plan of the second phase (after the new-cell list is complete).
-static __global__ void kb_plan_back(DomRec* recs, BatchPlan pl) {
-  block_prefix(pl.n, pl.all, [&](int k) {
-    return round32(recs[k].d.counts[recs[k].parity] + recs[k].d.counts[2]);
-  });
 }
 
 template <int Q, class S>
@@ -1754,10 +1383,6 @@ __global__ void __launch_bounds__(kGeoBlock, kGeoMinBlocks) kb_geometry(const Do
   }
 }
 
-// The batch's bulk hand-out counter: the int after the four prefix arrays
-// of the plan (n + 1 entries each), cleared by kb_plan_front every step.
-__device__ __forceinline__ int* batch_bulk_ctr(const BatchPlan& pl) { return pl.all + pl.n + 1; }
-
 // Units of all domains handed out as in k_bulk.
 template <int Q, class S, int COLL>
 __device__ __forceinline__ void batch_bulk_sweep(const DomRec* __restrict__ recs, const BatchPlan& pl) {
@@ -1767,7 +1392,7 @@ __device__ __forceinline__ void batch_bulk_sweep(const DomRec* __restrict__ recs
     const DomRec& r = recs[k];
     bulk_unit<Q, S, COLL>(r.d, r.p, r.parity, w - pl.bulk[k], r.d.counts[5]);
   };
-  hand_out_units<S>(total, batch_bulk_ctr(pl), unit);
+  hand_out_units<S>(total, &pl.ctr[0], unit);
 }
 
 template <int Q, class S, int COLL>
@@ -1777,8 +1402,8 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
 }
 
 // The batch's bulk sweep with the geometry tiles of all domains folded in,
-// as k_bulk_geo: the blocks first take tiles from the plan's tile counter
-// (the int after the bulk hand-out counter), then bulk units.
+// as k_bulk_geo: the blocks first take tiles from the plan's tile counter,
+// then bulk units.
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     kb_bulk_geo(const DomRec* __restrict__ recs, BatchPlan pl) {
@@ -1788,7 +1413,7 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     const int total = pl.tiles[pl.n];
     for (;;) {
       __syncthreads();  // every thread has read the previous s_tile
-      if (threadIdx.x == 0) s_tile = atomicAdd(batch_bulk_ctr(pl) + 1, 1);
+      if (threadIdx.x == 0) s_tile = atomicAdd(&pl.ctr[1], 1);
       __syncthreads();
       const int t = s_tile;
       if (t >= total) break;
@@ -1814,48 +1439,23 @@ __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) kb_interfa
   }
 }
 
-template <int Q>
-__global__ void __launch_bounds__(kBlock) kb_resolve(const DomRec* __restrict__ recs, BatchPlan pl) {
-  const int total = pl.band[pl.n];
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-    const int k = find_domain(pl.band, pl.n, g);
-    const DomRec& r = recs[k];
-    const int i = g - pl.band[k];
-    if (i < r.d.counts[r.parity]) resolve_cell<Q>(r.d, r.p, r.parity, i);
-  }
-}
-
-template <int Q>
-__global__ void __launch_bounds__(kBlock) kb_count(const DomRec* __restrict__ recs, BatchPlan pl) {
-  const int total = pl.band[pl.n];
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-    const int k = find_domain(pl.band, pl.n, g);
-    const DomRec& r = recs[k];
-    const int i = g - pl.band[k];
-    if (i < r.d.counts[r.parity]) count_cell<Q>(r.d, r.p, r.parity, i);
-  }
-}
-
-template <int Q, class S>
-__global__ void __launch_bounds__(128) kb_apply(const DomRec* __restrict__ recs, BatchPlan pl) {
-  const int total = pl.all[pl.n];
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-    const int k = find_domain(pl.all, pl.n, g);
-    const DomRec& r = recs[k];
-    const int i = g - pl.all[k];
-    if (i < r.d.counts[r.parity] + r.d.counts[2]) apply_cell<Q, S>(r.d, r.p, r.parity, i);
-  }
-}
-
 static __global__ void __launch_bounds__(kBlock) kb_finalize(const DomRec* __restrict__ recs, BatchPlan pl) {
-  const int total = pl.all[pl.n];
+  const int total = pl.band[pl.n];
+  const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   for (int base = wid * 32; base < total; base += warps * 32) {
-    const int k = find_domain(pl.all, pl.n, base);
+    const int k = find_domain(pl.band, pl.n, base);
     const DomRec& r = recs[k];
-    finalize_warp(r.d, r.p, r.parity, base - pl.all[k]);
+    const int i = base - pl.band[k] + lane;
+    finalize_lane(r.d, r.p, r.parity, i < r.d.counts[r.parity] ? r.d.band[r.parity][i] : -1, true);
   }
+  deal_domains(pl.n, [&](int k, int first, int stride) {
+    const DomRec& r = recs[k];
+    const int nnew = r.d.counts[2];
+    for (int b = first * 32; b < nnew; b += stride * 32)
+      finalize_lane(r.d, r.p, r.parity, b + lane < nnew ? r.d.newlist[b + lane] : -1, false);
+  });
 }
 
 // Bubble pressures of every domain (one block each), then the step is done
