@@ -277,7 +277,9 @@ fslbm_status fslbm_create(const fslbm_domain* domain, fslbm_lattice lattice,
   ALLOC(d.mom_u, 3 * N * rs);
   ALLOC(d.m_next, N * sizeof(double));
   ALLOC(d.phi_next, N * sizeof(double));
-  ALLOC(d.rho_band, N * sizeof(double));
+  // only the deviation formats keep the float fill levels, only FP64 rho_band
+  if (rs == 4) ALLOC(d.phif, N * sizeof(float));
+  if (rs == 8) ALLOC(d.rho_band, N * sizeof(double));
   ALLOC(d.err, 4 * sizeof(int));
   d.red_blocks = sms * 2;
   ALLOC(d.red, (size_t)d.red_blocks * kObsFields * sizeof(double));
@@ -1015,6 +1017,7 @@ fslbm_status fslbm_load(fslbm_ctx* c, const void* buf, size_t size) {
     e = cudaMemsetAsync(c->d.tile_mark, 0, nt * sizeof(int), c->stream);
   }
   if (e == cudaSuccess) {
+    k_derive_fields<<<(c->kp.N + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(c->d, c->kp);
     k_compact_full<<<(c->kp.N + kBlock - 1) / kBlock, kBlock, 0, c->stream>>>(c->d.flags, c->kp.N,
                                                                              c->d.band[0], &c->d.counts[0]);
     k_tiles_of_band<<<c->band_grid, kBlock, 0, c->stream>>>(c->d, c->kp, 0);

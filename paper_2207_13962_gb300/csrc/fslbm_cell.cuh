@@ -64,6 +64,14 @@ __device__ __forceinline__ int warp_append(int* counter, bool pred) {
   return pred ? base + __popc(b & ((1u << lane) - 1u)) : -1;
 }
 
+// Stores the fill level of a cell (and its float copy where the engine
+// keeps one: the conversion is then done once a store, not once a reader;
+// it runs on the integer pipe, see d2f).
+__device__ __forceinline__ void set_phi(const DPtrs& d, int c, double v) {
+  d.phi[c] = v;
+  if (d.phif) d.phif[c] = d2f(v);
+}
+
 // Largest domain k < n with off[k] <= g (off non-decreasing, off[0] = 0).
 __device__ __forceinline__ int find_domain(const int* __restrict__ off, int n, int g) {
   int lo = 0, hi = n;

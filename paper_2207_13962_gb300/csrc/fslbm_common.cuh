@@ -376,9 +376,14 @@ struct DPtrs {
                        // cell (static); sources outside the domain are not
                        // included
   double* phi;
+  float* phif;     // phi rounded to float (FP32 and 16-bit engines): what the
+                   // geometry and the mass exchange read of their neighbours;
+                   // written wherever phi is (set_phi)
   double* mass;
   int* bid;
-  uint8_t* cls;
+  uint8_t* cls;    // cell type, and in bits 2-3 the Thuerey class of an
+                   // interface cell: all the interface kernel reads of a
+                   // neighbour's kind
   uint8_t* mark;
   uint8_t* conv;
   uint8_t* cfin;

@@ -164,7 +164,7 @@ __device__ __forceinline__ void resolve_listed(const DPtrs& d, const KParams& p,
 __device__ __forceinline__ void commit_cell(const DPtrs& d, int parity, int k) {
   const int c = d.band[parity][k];
   d.mass[c] = d.m_next[k] + 0.0;
-  d.phi[c] = d.phi_next[k] + 0.0;
+  set_phi(d, c, d.phi_next[k] + 0.0);
 }
 
 // Excess-mass receivers (Eq. nm-fslbm-excess-mass) of list entry j:
@@ -218,7 +218,7 @@ __device__ __forceinline__ void apply_receiver(const DPtrs& d, const KParams& p,
   if (l.i == 0) {
     const double m = d.mass[c] + s;
     d.mass[c] = m;
-    d.phi[c] = m / band_rho<S>(d, c);
+    set_phi(d, c, m / band_rho<S>(d, c));
   }
 }
 
@@ -227,10 +227,10 @@ template <class S>
 __device__ __forceinline__ void apply_converted(const DPtrs& d, int c) {
   const uint8_t f = d.cfin[c];
   if (f == CV_TOL) {
-    d.phi[c] = 1.0;
+    set_phi(d, c, 1.0);
     d.mass[c] = band_rho<S>(d, c);
   } else if (f == CV_TOG) {
-    d.phi[c] = 0.0;
+    set_phi(d, c, 0.0);
     d.mass[c] = 0.0;
   }
 }
@@ -358,7 +358,7 @@ __device__ __forceinline__ void apply_new(const DPtrs& d, const KParams& p, int 
     if (l.i == 0) {
       const double m = 0.0 + s;
       d.mass[c] = m;
-      d.phi[c] = m / rb;
+      set_phi(d, c, m / rb);
     }
   } else {  // from liquid
     const bool gas_after = (t == T_GAS && !claimed) || (t == T_IFACE && cf == CV_TOG);
@@ -387,7 +387,7 @@ __device__ __forceinline__ void apply_new(const DPtrs& d, const KParams& p, int 
     if (l.i == 0) {
       const double m = rn + s;
       d.mass[c] = m;
-      d.phi[c] = m / rn;
+      set_phi(d, c, m / rn);
       d.bid[c] = best == 0xffffffffu ? -1 : (int)best;
     }
   }

@@ -77,9 +77,9 @@ __global__ void k_init_cells(const uint8_t* __restrict__ raw, const double* __re
   d.flags[c] = fl;
   d.wallmask[c] = wm;
   const double r = den ? den[c] : 1.0;
-  d.phi[c] = (t == T_LIQ) ? 1.0 : (t == T_IFACE) ? fill[c] : 0.0;
+  set_phi(d, c, (t == T_LIQ) ? 1.0 : (t == T_IFACE) ? fill[c] : 0.0);
   d.mass[c] = (t == T_LIQ) ? r : (t == T_IFACE) ? fill[c] * r : 0.0;
-  d.cls[c] = 0;
+  d.cls[c] = t;
   d.mark[c] = 0;
   d.conv[c] = 0;
   d.cfin[c] = 0;
@@ -467,7 +467,7 @@ __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, 
           if (X >= 0 && Y >= 0 && Z >= 0) {
             const int c = cidx(p, X, Y, Z);
             tv[q] = d.flags[c] & F_TYPE;
-            if constexpr (sizeof(R) == 4) pv[q] = d2f(d.phi[c]);
+            if constexpr (sizeof(R) == 4) pv[q] = d.phif[c];
             else pv[q] = d.phi[c];
           }
         }
@@ -737,7 +737,7 @@ __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, 
         hl |= (t == T_LIQ);
         hg |= (t == T_GAS);
       }
-      d.cls[c] = (!hl && hg) ? CL_NF : (hl && !hg) ? CL_NE : CL_STD;
+      d.cls[c] = T_IFACE | (((!hl && hg) ? CL_NF : (hl && !hg) ? CL_NE : CL_STD) << 2);
     }
     if (threadIdx.x == 0) d.tile_mark[tile] = 0;
   }
@@ -841,49 +841,69 @@ __device__ __forceinline__ void interface_cell(const DPtrs& d, const KParams& p,
   const R* rhog = (const R*)d.rhog;
 
     const int c = band[k];
-    int x, y, z;
-    decode(p, c, x, y, z);
-    // neighbours x + c_i and their types (independent loads issued together);
-    // the pull source of direction i is the neighbour in direction ibar.  A
-    // cell beside a free-slip face links to the mirror image of a neighbour
-    // across it, whose PDF arrives with the wall-normal component reversed.
-    const bool slipface = coll_slip(COLL) && (flags[c] & F_FACE) && (p.slip[0] | p.slip[1] | p.slip[2]);
+    const uint8_t fl = flags[c];
+    const uint32_t wm = (fl & F_NEAR_WALL) ? d.wallmask[c] : 0u;
+    // neighbours x + c_i (-1 outside the domain); the pull source of
+    // direction i is the neighbour in direction ibar.  A cell beside a
+    // free-slip face links to the mirror image of a neighbour across it,
+    // whose PDF arrives with the wall-normal component reversed.
+    const bool slipface = coll_slip(COLL) && (fl & F_FACE) && (p.slip[0] | p.slip[1] | p.slip[2]);
+    int x = 0, y = 0, z = 0;
     int nid[Q];
-    int nt[Q];
     nid[0] = c;
-    nt[0] = T_IFACE;
-    if (!slipface) {
+    if (!(fl & (F_FACE | F_WRAP))) {
 #pragma unroll
-      for (int i = 1; i < Q; ++i) nid[i] = nbr(p, x, y, z, CX(i), CY(i), CZ(i));
+      for (int i = 1; i < Q; ++i) nid[i] = c + p.off[i];
     } else {
+      decode(p, c, x, y, z);
+      if (!slipface) {
 #pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        int j;
-        bool mir;
-        nid[i] = pull_source<Q>(p, x, y, z, OPP(i), j, mir);
+        for (int i = 1; i < Q; ++i) nid[i] = nbr(p, x, y, z, CX(i), CY(i), CZ(i));
+      } else {
+#pragma unroll
+        for (int i = 1; i < Q; ++i) {
+          int j;
+          bool mir;
+          nid[i] = pull_source<Q>(p, x, y, z, OPP(i), j, mir);
+        }
       }
     }
-#pragma unroll
-    for (int i = 1; i < Q; ++i) nt[i] = ntype(flags, nid[i]);
+    // One level of loads: the neighbours' kind (type and class), fill level
+    // and arriving PDF do not depend on one another.  Which sources bounce
+    // back is static (the wall mask, or outside the domain; a mirror image
+    // that is an obstacle is told by its type), and what a gas neighbour's
+    // slot holds is dropped below.
     R fx[Q], f[Q];
-    unsigned miss = 0u;
+    int nt[Q];  // type, class in bits 2-3
+    nt[0] = T_IFACE;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) nt[i] = nid[i] >= 0 ? (int)d.cls[nid[i]] : (int)T_OBST;
 #pragma unroll
     for (int i = 0; i < Q; ++i) fx[i] = load_own<Q, S>(A, Np, c, i);
     f[0] = fx[0];  // the rest PDF stays in the cell
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-      const int st = nt[OPP(i)];
       const int src = nid[OPP(i)];
-      if (st == T_GAS) miss |= 1u << i;
-      const bool fluid = (st == T_LIQ || st == T_IFACE);
-      int j = i;  // the PDF that arrives in direction i
-      if (slipface) {
+      if (!slipface) {
+        // A[i Np + src]: with the neighbour at c - off[i] its offset is the
+        // interior one
+        const bool own = src < 0 || ((wm >> i) & 1u);
+        f[i] = load_w<S, Q>(A[(long long)(own ? OPP(i) : i) * Np + (own ? c : src)], i);
+      } else {
+        int j;
         bool mir;
         (void)pull_source<Q>(p, x, y, z, i, j, mir);
+        const bool own = (nt[OPP(i)] & 3) == T_OBST;
+        f[i] = load_w<S, Q>(A[(long long)(own ? OPP(i) : j) * Np + (own ? c : src)], i);
       }
-      const T v = A[(long long)(fluid ? j : OPP(i)) * Np + (fluid ? src : c)];
-      f[i] = load_w<S, Q>(v, i);
-      if (st == T_GAS) f[i] = R(0.0);
+    }
+    unsigned miss = 0u;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      if ((nt[OPP(i)] & 3) == T_GAS) {
+        miss |= 1u << i;
+        f[i] = R(0.0);
+      }
     }
     // mass exchange with the streamed (not yet reconstructed) PDFs:
     // a = f*_ibar(x + c_i) equals the pulled f_ibar(x).  With deviations
@@ -891,63 +911,69 @@ __device__ __forceinline__ void interface_cell(const DPtrs& d, const KParams& p,
     // float pair, so a liquid neighbour's PDF sum changes by exactly -dm_i;
     // an interface link's term is the float product of the same operands
     // that the neighbour negates, so the two terms cancel exactly.
-    const double phic = d.phi[c];
-    const int clc = d.cls[c];
+    const int clc = d.cls[c] >> 2;
     double dm = 0.0;
-    FAcc acc;
-    const float phicf = d2f(phic);
-    // class and fill level of the interface neighbours, read a chunk of
-    // directions at a time ahead of the (ordered) accumulation
-    constexpr int kChunk = kIfaceChunk;
+    if constexpr (S::kDev) {
+      FAcc acc;
+      const float phicf = d.phif[c];
+      float phn[Q];
 #pragma unroll
-    for (int i0 = 1; i0 < Q; i0 += kChunk) {
-      int cl9[kChunk];
-      double ph9[kChunk];
+      for (int i = 1; i < Q; ++i) phn[i] = nid[i] >= 0 ? d.phif[nid[i]] : 0.0f;
 #pragma unroll
-      for (int a = 0; a < kChunk; ++a) {
-        const int i = i0 + a;
-        if (i < Q && nt[i] == T_IFACE) {
-          cl9[a] = d.cls[nid[i]];
-          ph9[a] = d.phi[nid[i]];
+      for (int i = 1; i < Q; ++i) {
+        const int ntp = nt[i] & 3;
+        if (ntp == T_GAS || ntp == T_OBST) continue;
+        const float fa = f[OPP(i)];
+        const float fb = fx[i];
+        if (ntp == T_LIQ) {
+          acc.add_diff(fa, fb);
+        } else {
+          const float w = W<Q, float>(i);
+          const int cln = nt[i] >> 2;
+          float v;
+          if (clc == cln) v = __fsub_rn(fa, fb);
+          else if (clc == CL_STD) v = (cln == CL_NF) ? __fadd_rn(fa, w) : -__fadd_rn(fb, w);
+          else if (clc == CL_NF) v = -__fadd_rn(fb, w);
+          else v = __fadd_rn(fa, w);
+          acc.add(__fmul_rn(__fmul_rn(0.5f, __fadd_rn(phicf, phn[i])), v));
         }
       }
+      dm = acc.value();
+    } else {
+      const double phic = d.phi[c];
+      // the interface neighbours' fill levels, read a chunk of directions at
+      // a time ahead of the (ordered) accumulation
+      constexpr int kChunk = kIfaceChunk;
 #pragma unroll
-      for (int a = 0; a < kChunk; ++a) {
-        const int i = i0 + a;
-        if (i >= Q) continue;
-        const int ntp = nt[i];
-        if (ntp == T_GAS || ntp == T_OBST) continue;
-        const R fa = f[OPP(i)];
-        const R fb = fx[i];
-        if constexpr (S::kDev) {
-          const float w = W<Q, float>(i);
-          if (ntp == T_LIQ) {
-            acc.add_diff(fa, fb);
-          } else {
-            const int cln = cl9[a];
-            float v;
-            if (clc == cln) v = __fsub_rn(fa, fb);
-            else if (clc == CL_STD) v = (cln == CL_NF) ? __fadd_rn(fa, w) : -__fadd_rn(fb, w);
-            else if (clc == CL_NF) v = -__fadd_rn(fb, w);
-            else v = __fadd_rn(fa, w);
-            acc.add(__fmul_rn(__fmul_rn(0.5f, __fadd_rn(phicf, d2f(ph9[a]))), v));
-          }
-        } else {
+      for (int i0 = 1; i0 < Q; i0 += kChunk) {
+        double ph[kChunk];
+#pragma unroll
+        for (int a = 0; a < kChunk; ++a) {
+          const int i = i0 + a;
+          ph[a] = i < Q && nid[i] >= 0 ? d.phi[nid[i]] : 0.0;
+        }
+#pragma unroll
+        for (int a = 0; a < kChunk; ++a) {
+          const int i = i0 + a;
+          if (i >= Q) continue;
+          const int ntp = nt[i] & 3;
+          if (ntp == T_GAS || ntp == T_OBST) continue;
+          const R fa = f[OPP(i)];
+          const R fb = fx[i];
           if (ntp == T_LIQ) {
             dm = dm + (double)(fa - fb);
           } else {
-            const int cln = cl9[a];
+            const int cln = nt[i] >> 2;
             R v;
             if (clc == cln) v = fa - fb;
             else if (clc == CL_STD) v = (cln == CL_NF) ? fa : -fb;
             else if (clc == CL_NF) v = -fb;
             else v = fa;
-            dm = dm + 0.5 * (phic + ph9[a]) * (double)v;
+            dm = dm + 0.5 * (phic + ph[a]) * (double)v;
           }
         }
       }
     }
-    if constexpr (S::kDev) dm = acc.value();
     const double mn = d.mass[c] + dm;
     // BC velocity from the cell's own post-collision PDFs
     R rc, jx, jy, jz;
@@ -1039,8 +1065,7 @@ __device__ __forceinline__ void interface_cell(const DPtrs& d, const KParams& p,
       mu_out[3LL * c + 2] = mu[2];
     }
     {
-      const uint8_t fl = flags[c];
-      if (fl & F_NEAR_WALL) write_reflected<Q, S>(d, p, B, c, d.wallmask[c], (fl & F_WRAP) != 0, f);
+      if (fl & F_NEAR_WALL) write_reflected<Q, S>(d, p, B, c, wm, (fl & F_WRAP) != 0, f);
     }
     double phin;
     if constexpr (S::kDev) {
@@ -1061,11 +1086,20 @@ __device__ __forceinline__ void interface_cell(const DPtrs& d, const KParams& p,
     if (mark != CV_NONE) append_conversion(d, parity, c);
   }
 
+// List entry that a thread of the grid starts at.  A list that needs at most
+// one warp of every block is dealt a warp a block, so that it spreads over
+// the SMs; a longer one runs through the blocks in order (neighbouring
+// entries are neighbouring cells, whose reads share the SM's L1).
+__device__ __forceinline__ int band_start(int n) {
+  if (n <= (int)gridDim.x * 32) return ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+  return blockIdx.x * blockDim.x + threadIdx.x;
+}
+
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) k_interface(DPtrs d, KParams p, int parity) {
   const int n = d.counts[parity];
   bool bad = false;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
+  for (int k = band_start(n); k < n; k += gridDim.x * blockDim.x)
     interface_cell<Q, S, COLL>(d, p, parity, k, bad);
   if (bad) d.err[0] = 1;
 }
@@ -1118,6 +1152,14 @@ static __global__ void k_segs_init(DPtrs d, KParams p) {
   if (fresh) d.segs[pos] = c / kSegCells;
 }
 
+// What the context derives from flags and fill levels (checkpoint load).
+static __global__ void k_derive_fields(DPtrs d, KParams p) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= p.N) return;
+  d.cls[c] = d.flags[c] & F_TYPE;
+  if (d.phif) d.phif[c] = d2f(d.phi[c]);
+}
+
 // Tile list of an interface list (initial state and checkpoint load).
 static __global__ void k_tiles_of_band(DPtrs d, KParams p, int parity) {
   const int n = d.counts[parity];
@@ -1150,10 +1192,12 @@ __device__ __forceinline__ void finalize_lane(const DPtrs& d, const KParams& p, 
       }
       if (f == CV_TOL) {
         d.flags[c] = (fl & ~F_TYPE) | T_LIQ;
+        d.cls[c] = T_LIQ;
         d.bid[c] = -1;
         to_liq = true;
       } else if (f == CV_TOG) {
         d.flags[c] = (fl & ~F_TYPE) | T_GAS;
+        d.cls[c] = T_GAS;
         dgas = 1;
       } else {
         keep = true;
@@ -1161,6 +1205,7 @@ __device__ __forceinline__ void finalize_lane(const DPtrs& d, const KParams& p, 
     } else {
       if ((fl & F_TYPE) == T_GAS) dgas = -1;
       d.flags[c] = (fl & ~F_TYPE) | T_IFACE;
+      d.cls[c] = T_IFACE;  // its class follows with the next geometry pass
       d.claim[c] = 0;
       keep = true;
     }
@@ -1428,7 +1473,7 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) kb_interface(const DomRec* __restrict__ recs, BatchPlan pl) {
   const int total = pl.band[pl.n];
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
+  for (int g = band_start(total); g < total; g += gridDim.x * blockDim.x) {
     const int k = find_domain(pl.band, pl.n, g);
     const DomRec& r = recs[k];
     const int i = g - pl.band[k];
