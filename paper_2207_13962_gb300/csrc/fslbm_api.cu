@@ -281,7 +281,7 @@ fslbm_status fslbm_create(const fslbm_domain* domain, fslbm_lattice lattice,
   if (rs == 4) ALLOC(d.phif, N * sizeof(float));
   if (rs == 8) ALLOC(d.rho_band, N * sizeof(double));
   ALLOC(d.err, 4 * sizeof(int));
-  d.red_blocks = sms * 2;
+  d.red_blocks = sms * kObsBlocksPerSm;
   ALLOC(d.red, (size_t)d.red_blocks * kObsFields * sizeof(double));
   ALLOC(c->d_obs, kObsFields * sizeof(double));
 #undef ALLOC

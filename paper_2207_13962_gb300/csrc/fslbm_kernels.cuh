@@ -1267,40 +1267,113 @@ __device__ __forceinline__ void bubble_update(const DPtrs& d, const KParams& p) 
 static __global__ void k_bubble(DPtrs d, KParams p) { bubble_update(d, p); }
 
 // ------------------------------------------------------------ observables
-// Per-block partials: [0] mass, [1] max|u|, [2] liquid volume, [3] nan,
+// Per-block partials: [0] mass, [1] max|u|^2, [2] liquid volume, [3] nan,
 // [4..7] counts of gas, interface, liquid, obstacle.
+//
+// One read of the PDFs bounds the pass if the FP64 unit (two lanes a clock
+// per SM) is kept out of it, so the deviation formats do their per-cell work
+// in FP32: rho - 1 is summed as a float pair (or in grid steps), u and the
+// candidates for the largest |u| are formed in FP32, and FP64 squares only
+// where the FP32 estimate comes near the largest value so far (the result is
+// the FP64 one).  The mass is the number of liquid cells plus the FP64 sum of
+// their deviations plus the interface masses; |u| is rooted once, at the end.
+// 160x160x512 tube, FP32 (8.2 M fluid cells, 0.65 GB): 1000 us with FP64
+// moments and 2 blocks per SM.
 constexpr int kObsFields = 8;
+constexpr int kObsBlocksPerSm = 4;
 
+// rho - 1 of a cell in FP64, rho in FP32 and the velocity, for the
+// observables (the velocity in post_moments' arithmetic).
 template <int Q, class S>
-__global__ void __launch_bounds__(kBlock) k_obs_partial(DPtrs d, KParams p, int parity,
-                                                        double* part) {
+__device__ __forceinline__ void obs_moments(const typename S::T* P, long long Np, int c, const KParams& p,
+                                            double& dr, float& rr, float u[3]) {
+  float f[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) f[i] = load_own<Q, S>(P, Np, c, i);
+  float r, jx, jy, jz;
+  sums<Q, float>(f, r, jx, jy, jz);
+  if constexpr (S::kExactRest) {
+    int n0 = rest_slice<Q, S>(P, Np)[c];
+    long long n = n0;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) n += grid_steps32<S>(f[i]);  // f[i] is a stored value
+    dr = (double)n * (1.0 / (double)(1LL << S::kShift));
+    rr = d2f(1.0 + dr);
+  } else {
+    FAcc a;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) a.add(f[i]);
+    dr = a.value();
+    // rho rounded to float, from the pair
+    const float lo = a.lo;
+    a.lo = 0.f;
+    a.add(1.0f);
+    rr = a.hi + (a.lo + lo);
+  }
+  u[0] = jx / rr - 0.5f * gpar<float>(p, 0);
+  u[1] = jy / rr - 0.5f * gpar<float>(p, 1);
+  u[2] = jz / rr - 0.5f * gpar<float>(p, 2);
+}
+
+// kOwn: the state is a context's (liquid cells have fill level 1); otherwise
+// the arrays are a caller's.
+template <int Q, class S, bool kOwn>
+__global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d, KParams p, int parity,
+                                                                          double* part) {
   using R = typename S::Real;
   const typename S::T* P = (const typename S::T*)d.pdf[parity];
-  // the mass is summed per thread with Neumaier's compensation, then
-  // pairwise across threads and blocks
-  double mass = 0.0, mcomp = 0.0, umax = 0.0, vol = 0.0, nan = 0.0, cnt[4] = {0, 0, 0, 0};
+  // interface masses (and all masses in FP64) are summed per thread with
+  // Neumaier's compensation, then pairwise across threads and blocks
+  double mass = 0.0, mcomp = 0.0, dev = 0.0, u2max = 0.0, vol = 0.0;
+  float near_max = -1.0f;  // a float bound below the largest |u|^2 so far
+  int nan = 0, cnt[4] = {0, 0, 0, 0};
+  auto add_mass = [&](double x) {
+    const double s = mass + x;
+    mcomp += (fabs(mass) >= fabs(x)) ? ((mass - s) + x) : ((x - s) + mass);
+    mass = s;
+  };
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < p.N; c += gridDim.x * blockDim.x) {
     const int t = d.flags[c] & F_TYPE;
-    cnt[t] += 1.0;
-    if (t == T_LIQ || t == T_IFACE) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) cnt[k] += t == k;
+    if (t != T_LIQ && t != T_IFACE) continue;
+    double m = 0.0;
+    if (!kOwn || !S::kDev || t == T_IFACE) {
+      m = d.mass[c];
+      if (!(m == m)) nan = 1;
+    }
+    if (!kOwn || t == T_IFACE) vol += d.phi[c];
+    if constexpr (S::kDev) {
+      double dr;
+      float rr, u[3];
+      obs_moments<Q, S>(P, p.Np, c, p, dr, rr, u);
+      const float q = __fmaf_rn(u[0], u[0], __fmaf_rn(u[1], u[1], u[2] * u[2]));
+      if (!(q == q) || !(rr > 0.0f)) nan = 1;
+      if (q >= near_max) {
+        const double uu = (double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2];
+        if (uu > u2max) u2max = uu;
+        near_max = (float)u2max * 0.9999f;
+      }
+      if (t == T_LIQ) dev += dr;
+      else add_mass(m);
+    } else {
       double r;
       R u[3];
       post_moments<Q, S>(P, p.Np, c, p, r, u);
-      const double uu = sqrt((double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2]);
-      if (!(uu == uu) || !(r > 0.0)) nan = 1.0;
-      if (uu > umax) umax = uu;
-      {
-        const double x = (t == T_LIQ) ? r : d.mass[c];
-        const double s = mass + x;
-        mcomp += (fabs(mass) >= fabs(x)) ? ((mass - s) + x) : ((x - s) + mass);
-        mass = s;
-      }
-      vol += d.phi[c];
-      if (!(d.mass[c] == d.mass[c])) nan = 1.0;
+      const double uu = (double)u[0] * u[0] + (double)u[1] * u[1] + (double)u[2] * u[2];
+      if (!(uu == uu) || !(r > 0.0)) nan = 1;
+      if (uu > u2max) u2max = uu;
+      add_mass((t == T_LIQ) ? r : m);
     }
   }
+  if constexpr (S::kDev) {
+    add_mass(dev);
+    add_mass((double)cnt[T_LIQ]);
+  }
+  if constexpr (kOwn) vol += (double)cnt[T_LIQ];
   __shared__ double sh[kObsFields][kBlock / 32];
-  double v[kObsFields] = {mass + mcomp, umax, vol, nan, cnt[0], cnt[1], cnt[2], cnt[3]};
+  double v[kObsFields] = {mass + mcomp, u2max, vol, (double)nan, (double)cnt[0], (double)cnt[1], (double)cnt[2],
+                          (double)cnt[3]};
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int f = 0; f < kObsFields; ++f) {
@@ -1320,15 +1393,22 @@ __global__ void __launch_bounds__(kBlock) k_obs_partial(DPtrs d, KParams p, int 
   }
 }
 
-static __global__ void k_obs_final(const double* part, int nblocks, double* out) {
-  const int f = threadIdx.x;
-  if (f >= kObsFields) return;
-  double a = part[f];
-  for (int b = 1; b < nblocks; ++b) {
+// One warp a field: each lane adds every 32nd partial, then the lanes add up
+// (a single thread a field reads the partials one after another: 46 us for
+// 304 blocks).
+static __global__ void __launch_bounds__(32 * kObsFields) k_obs_final(const double* part, int nblocks, double* out) {
+  const int f = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool mx = f == 1 || f == 3;
+  double a = 0.0;  // of a sum and of maxima of values >= 0
+  for (int b = lane; b < nblocks; b += 32) {
     const double v = part[b * kObsFields + f];
-    a = (f == 1 || f == 3) ? fmax(a, v) : a + v;
+    a = mx ? fmax(a, v) : a + v;
   }
-  out[f] = a;
+  for (int o = 16; o > 0; o >>= 1) {
+    const double b = __shfl_down_sync(0xffffffffu, a, o);
+    a = mx ? fmax(a, b) : a + b;
+  }
+  if (lane == 0) out[f] = f == 1 ? sqrt(a) : a;
 }
 
 // PDFs of the current buffer as FP64 (zero on gas and obstacle cells), in
