@@ -373,17 +373,26 @@ __device__ __forceinline__ R k8w(int n2) {
 
 // Geometry on 8^3 tiles that hold interface cells (tile list built by
 // k_finalize).  The tile's fill levels with a halo of 3 sit in shared memory;
-// phi~ (K8 smoothing, radius 2) is formed on the 12^3 sub-box, n^ (Parker-
-// Youngs, Eq. nm-fslbm-normal) on the 10^3 sub-box and kappa = -div(n^) on
-// the interface cells of the tile.  Obstacle and out-of-domain stencil
-// points take the stencil centre's value.  In the FP64 engine each value
-// uses the same arithmetic and summation order as a per-cell evaluation.
+// phi~ (K8 smoothing, radius 2) lies on the 12^3 sub-box, n^ (Parker-Youngs,
+// Eq. nm-fslbm-normal) on the 10^3 sub-box and kappa = -div(n^) on the
+// interface cells of the tile.  Obstacle and out-of-domain stencil points
+// take the stencil centre's value.  In the FP64 engine each value uses the
+// same arithmetic and summation order as a per-cell evaluation.
+//
+// An interface is a sheet: kappa needs n^ at the interface cells and their
+// face neighbours only, and these need phi~ on the 3^3 blocks around them,
+// together about a third of the sub-boxes.  The points needed are marked as
+// the box is loaded, compacted into two lists in shared memory and evaluated
+// a thread a point, so the work follows the interface and fills the warps.
+// Marching all z-columns of the sub-boxes instead (144 and 100 threads, 12
+// and 10 steps) measured 99 us for the six tiles of the 32x64x1 wave in FP64,
+// where the FP64 pipe of one SM (two lanes a clock) bounds a tile.
 constexpr int GT = 8;                    // tile edge
 constexpr int GE = GT + 6;               // box edge with halo 3
 constexpr int GB = GE * GE * GE;         // 2744 box positions
 constexpr int GS = GT + 4;               // phi~ sub-box edge (12)
 constexpr int GN = GT + 2;               // n^ sub-box edge (10)
-constexpr int kGeoBlock = 192;  // the z-column phases use 144 and 100 threads
+constexpr int kGeoBlock = 256;
 #ifndef FSLBM_GEO_LOAD_BATCH
 #define FSLBM_GEO_LOAD_BATCH 6
 #endif
@@ -407,12 +416,162 @@ template <class R>
 __device__ __forceinline__ bool is_obstacle(R v) { return v < R(-1.0e29); }
 
 // Shared memory of one tile: the fill-level box, whose space the normals
-// take over once the smoothing has read it, the smoothed sub-box and the
-// types.
-constexpr int kGeoBoxSlots = GB > 3 * GN * GN * GN ? GB : 3 * GN * GN * GN;
+// take over once the smoothing has read it; the smoothed sub-box, whose space
+// holds the marks of the needed points until the lists are made; the types;
+// the lists.
+constexpr int GN3 = GN * GN * GN, GS3 = GS * GS * GS;
+constexpr int kGeoBoxSlots = GB > 3 * GN3 ? GB : 3 * GN3;
 template <class R>
 constexpr size_t geometry_smem() {
-  return sizeof(R) * (kGeoBoxSlots + GS * GS * GS) + GB;
+  return sizeof(R) * (kGeoBoxSlots + GS3) + GB + sizeof(unsigned short) * (GN3 + GS3);
+}
+static_assert(GN3 + GS3 <= 4 * GS3 && GN3 % 4 == 0 && GS3 % 4 == 0 && GB % 8 == 0, "layout of the tile's buffers");
+
+// a / 3.6796875 (= 471 / 128, the sum of the K8 weights), correctly rounded:
+// fma(a, zh, a zl) with zh + zl = 128 / 471 to twice the precision (Brisebarre,
+// Muller and Raina, "Accelerating correctly rounded floating-point division
+// when the divisor is known in advance", IEEE Trans. Computers 53, 2004).  A
+// quotient by 471 of a binary number lies at least 1/942 of an ulp from any
+// midpoint of two neighbouring numbers, and the sum before its rounding is
+// within 2^-51 ulp of the quotient, so the rounding is that of the division.
+__device__ __forceinline__ double div_k8(double a) {
+  return fma(a, 0x1.1648d50fc3201p-2, a * 0x1.648d50fc32011p-58);
+}
+
+// Warp-wide append to a list in shared memory; every lane calls it.
+__device__ __forceinline__ void push_shared(unsigned short* list, int* count, bool take, int value) {
+  const unsigned m = __ballot_sync(0xffffffffu, take);
+  if (!m) return;
+  const unsigned lane = threadIdx.x & 31u;
+  int base = 0;
+  if (lane == 0) base = atomicAdd(count, __popc(m));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (take) list[base + __popc(m & ((1u << lane) - 1u))] = (unsigned short)value;
+}
+
+// phi~ at box position b (not an obstacle).  The FP32 engines group the 27
+// points by z-plane: the K8 weights depend on r^2 only, so a plane gives its
+// centre, the sum of its 4 in-plane face neighbours and of its 4 corners; an
+// obstacle point takes the value of the stencil's centre, so a plane keeps the
+// sum over its other points and, beside it, the count of its obstacle points,
+// which multiplies the centre value at the end.  The FP64 engine sums in the
+// oracle's order; the weights 2^-4 and 2^-8 make exact products, so a fused
+// operation rounds as the product and the sum do.
+template <class R, bool kSolid>
+__device__ __forceinline__ R smoothed_at(const R* sphi, int b) {
+  const R* q = sphi + b;
+  const R pc = q[0];
+  if constexpr (sizeof(R) == 4) {
+    auto nz = [&](R v) { return (kSolid && is_obstacle(v)) ? R(0.0) : v; };
+    auto ob = [&](R v) { return (kSolid && is_obstacle(v)) ? R(1.0) : R(0.0); };
+    R c0[3], f4[3], c4[3], nf[3], nc[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const R* w = q + (k - 1) * GE * GE;
+      c0[k] = w[0];
+      const R a = w[-1], e = w[1], c = w[-GE], g = w[GE];
+      const R u = w[-GE - 1], v = w[-GE + 1], x = w[GE - 1], y = w[GE + 1];
+      f4[k] = (nz(a) + nz(e)) + (nz(c) + nz(g));
+      c4[k] = (nz(u) + nz(v)) + (nz(x) + nz(y));
+      if constexpr (kSolid) {
+        nf[k] = (ob(a) + ob(e)) + (ob(c) + ob(g));
+        nc[k] = (ob(u) + ob(v)) + (ob(x) + ob(y));
+      }
+    }
+    const R zm = (kSolid && is_obstacle(c0[0])) ? pc : c0[0], zp = (kSolid && is_obstacle(c0[2])) ? pc : c0[2];
+    R s1 = (f4[1] + zm) + zp, s2 = (c4[1] + f4[0]) + f4[2], s3 = c4[0] + c4[2];
+    if constexpr (kSolid) {
+      s1 = s1 + nf[1] * pc;
+      s2 = s2 + (nc[1] + nf[0] + nf[2]) * pc;
+      s3 = s3 + (nc[0] + nc[2]) * pc;
+    }
+    return (pc + k8w<R>(1) * s1 + k8w<R>(2) * s2 + k8w<R>(3) * s3) * (R(1.0) / R(3.6796875));
+  } else {
+    R acc = R(0.0);
+#pragma unroll
+    for (int dz = -1; dz <= 1; ++dz)
+#pragma unroll
+      for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+        for (int dx = -1; dx <= 1; ++dx) {
+          const int n2 = dx * dx + dy * dy + dz * dz;
+          const R raw = q[dx + GE * (dy + GE * dz)];
+          const R v = (kSolid && is_obstacle(raw)) ? pc : raw;
+          if (n2 == 0) acc = acc + v;
+          else if (n2 == 1) acc = acc + k8w<R>(1) * v;
+          else acc = fma(k8w<R>(n2), v, acc);
+        }
+    return div_k8(acc);
+  }
+}
+
+// n^ at position s of the smoothed sub-box (not an obstacle).  FP32: the
+// Parker-Youngs weights (2-|d|)(2-|d'|) factor into [1 2 1] x [1 2 1] x
+// [-1 0 1], formed per z-plane with the (weighted) obstacle counts beside them
+// as above.  FP64: the oracle's order; the weights 1, 2 and 4 make exact
+// products.
+template <class R, bool kSolid>
+__device__ __forceinline__ void normal_at(const R* sps, int s, R n[3]) {
+  const R* q = sps + s;
+  const R pc = q[0];
+  if constexpr (sizeof(R) == 4) {
+    auto nz = [&](R v) { return (kSolid && is_obstacle(v)) ? R(0.0) : v; };
+    auto ob = [&](R v) { return (kSolid && is_obstacle(v)) ? R(1.0) : R(0.0); };
+    R gx[3], gy[3], sm[3], gxo[3], gyo[3], so[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const R* w = q + (k - 1) * GS * GS;
+      const R a00 = w[-GS - 1], a01 = w[-GS], a02 = w[-GS + 1];
+      const R a10 = w[-1], a11 = w[0], a12 = w[1];
+      const R a20 = w[GS - 1], a21 = w[GS], a22 = w[GS + 1];
+      gx[k] = (nz(a02) - nz(a00)) + R(2.0) * (nz(a12) - nz(a10)) + (nz(a22) - nz(a20));
+      gy[k] = (nz(a20) - nz(a00)) + R(2.0) * (nz(a21) - nz(a01)) + (nz(a22) - nz(a02));
+      sm[k] = (nz(a00) + R(2.0) * nz(a01) + nz(a02)) + R(2.0) * (nz(a10) + R(2.0) * nz(a11) + nz(a12)) +
+              (nz(a20) + R(2.0) * nz(a21) + nz(a22));
+      if constexpr (kSolid) {
+        gxo[k] = (ob(a02) - ob(a00)) + R(2.0) * (ob(a12) - ob(a10)) + (ob(a22) - ob(a20));
+        gyo[k] = (ob(a20) - ob(a00)) + R(2.0) * (ob(a21) - ob(a01)) + (ob(a22) - ob(a02));
+        so[k] = (ob(a00) + R(2.0) * ob(a01) + ob(a02)) + R(2.0) * (ob(a10) + R(2.0) * ob(a11) + ob(a12)) +
+                (ob(a20) + R(2.0) * ob(a21) + ob(a22));
+      }
+    }
+    R n0 = gx[0] + R(2.0) * gx[1] + gx[2];
+    R n1 = gy[0] + R(2.0) * gy[1] + gy[2];
+    R n2 = sm[2] - sm[0];
+    if constexpr (kSolid) {
+      n0 = n0 + (gxo[0] + R(2.0) * gxo[1] + gxo[2]) * pc;
+      n1 = n1 + (gyo[0] + R(2.0) * gyo[1] + gyo[2]) * pc;
+      n2 = n2 + (so[2] - so[0]) * pc;
+    }
+    const R l2 = n0 * n0 + n1 * n1 + n2 * n2;
+    const R il = l2 > R(0.0) ? rsqrtf(l2) : R(0.0);
+    n[0] = n0 * il;
+    n[1] = n1 * il;
+    n[2] = n2 * il;
+  } else {
+    auto at = [&](int dx, int dy, int dz) { return q[dx + GS * (dy + GS * dz)]; };
+    R nn[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      R acc = R(0.0);
+#pragma unroll
+      for (int pp = -1; pp <= 1; ++pp)
+#pragma unroll
+        for (int r = -1; r <= 1; ++r) {
+          const int ax = (a == 0) ? 1 : r, ay = (a == 0) ? r : (a == 1) ? 1 : pp, az = (a == 2) ? 1 : pp;
+          const int bx = (a == 0) ? -1 : ax, by = (a == 1) ? -1 : ay, bz = (a == 2) ? -1 : az;
+          const R rp = at(ax, ay, az), rm = at(bx, by, bz);
+          const R vp = (kSolid && is_obstacle(rp)) ? pc : rp;
+          const R vm = (kSolid && is_obstacle(rm)) ? pc : rm;
+          const R wt = (pp == 0 && r == 0) ? R(4.0) : (pp == 0 || r == 0) ? R(2.0) : R(1.0);
+          acc = fma(wt, vp - vm, acc);
+        }
+      nn[a] = acc;
+    }
+    const R len = sqrt(nn[0] * nn[0] + nn[1] * nn[1] + nn[2] * nn[2]);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) n[a] = (len > R(0.0)) ? nn[a] / len : R(0.0);
+  }
 }
 
 // One 8^3 tile of the geometry pass (all NT threads of the block call it).
@@ -421,326 +580,183 @@ __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, 
                                               unsigned char* g_smem) {
   using R = typename S::Real;
   constexpr int kPer = (GB + NT - 1) / NT;  // box positions per thread
+  __shared__ int s_count[2];                // points in the lists
   R* sphi = (R*)g_smem;
   R* snh = sphi;  // written after the smoothing's last read of sphi
   R* sps = sphi + kGeoBoxSlots;
-  uint8_t* styp = (uint8_t*)(sps + GS * GS * GS);
+  uint8_t* need_n = (uint8_t*)sps;  // marks, until the lists are made
+  uint8_t* need_s = need_n + GN3;
+  uint8_t* styp = (uint8_t*)(sps + GS3);
+  unsigned short* list_n = (unsigned short*)(styp + GB);
+  unsigned short* list_s = list_n + GN3;
   const int ntx = (p.nx + GT - 1) / GT, nty = (p.ny + GT - 1) / GT;
   R* nhat = (R*)d.nhat;
   R* rhog = (R*)d.rhog;
-  const R wsum = R(3.6796875);
 
-    const int tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
-    const int ox = tx * GT - 3, oy = ty * GT - 3, oz = tz * GT - 3;
-    // all of a thread's global reads of the box are issued before the first
-    // shared-memory store (NT threads, kPer positions each)
-    __syncthreads();
-    // Thread t loads box position t + r NT counted in the cells'
-    // storage order (its first coordinate runs along the contiguous axis),
-    // so that the loads of a warp coalesce whatever the storage order; the
-    // shared-memory box itself is indexed in the caller's axes.
-    auto box_pos = [&](int b, int& i, int& j, int& k) {
-      const int k0 = b % GE, k1 = (b / GE) % GE, k2 = b / (GE * GE);
-      i = sel3(p.inv[0], k0, k1, k2);
-      j = sel3(p.inv[1], k0, k1, k2);
-      k = sel3(p.inv[2], k0, k1, k2);
-    };
-    // in kLoadRounds rounds of at most kBatch positions, so that the loads in
-    // flight fit the registers of a 64-register thread
-    constexpr int kBatch = kGeoLoadBatch < kPer ? kGeoLoadBatch : kPer;
-    bool solid_here = false;  // an obstacle or a position outside the domain
+  const int tx = tile % ntx, ty = (tile / ntx) % nty, tz = tile / (ntx * nty);
+  const int ox = tx * GT - 3, oy = ty * GT - 3, oz = tz * GT - 3;
+  __syncthreads();  // the previous tile is done with the buffers
+  for (int w = threadIdx.x; w < (GN3 + GS3) / 4; w += NT) ((unsigned*)need_n)[w] = 0u;
+  if (threadIdx.x < 2) s_count[threadIdx.x] = 0;
+  __syncthreads();
+  // Thread t loads box position t + r NT counted in the cells' storage order
+  // (its first coordinate runs along the contiguous axis), so that the loads
+  // of a warp coalesce whatever the storage order; the shared-memory box
+  // itself is indexed in the caller's axes.
+  auto box_pos = [&](int b, int& i, int& j, int& k) {
+    const int k0 = b % GE, k1 = (b / GE) % GE, k2 = b / (GE * GE);
+    i = sel3(p.inv[0], k0, k1, k2);
+    j = sel3(p.inv[1], k0, k1, k2);
+    k = sel3(p.inv[2], k0, k1, k2);
+  };
+  // in rounds of at most kBatch positions, all of whose global reads are
+  // issued before the first shared-memory store (the loads in flight fit the
+  // registers of a 64-register thread)
+  constexpr int kBatch = kGeoLoadBatch < kPer ? kGeoLoadBatch : kPer;
+  bool solid_here = false;  // an obstacle or a position outside the domain
 #pragma unroll
-    for (int r0 = 0; r0 < kPer; r0 += kBatch) {
-      uint8_t tv[kBatch];
-      R pv[kBatch];
+  for (int r0 = 0; r0 < kPer; r0 += kBatch) {
+    uint8_t tv[kBatch];
+    R pv[kBatch];
 #pragma unroll
-      for (int q = 0; q < kBatch; ++q) {
-        const int b = threadIdx.x + (r0 + q) * NT;
-        tv[q] = 4;  // outside the domain: solid
-        pv[q] = R(0.0);
-        if (r0 + q < kPer && b < GB) {
-          int i, j, k;
-          box_pos(b, i, j, k);
-          const int X = wrapc(ox + i, p.nx, p.per[0]);
-          const int Y = wrapc(oy + j, p.ny, p.per[1]);
-          const int Z = wrapc(oz + k, p.nz, p.per[2]);
-          if (X >= 0 && Y >= 0 && Z >= 0) {
-            const int c = cidx(p, X, Y, Z);
-            tv[q] = d.flags[c] & F_TYPE;
-            if constexpr (sizeof(R) == 4) pv[q] = d.phif[c];
-            else pv[q] = d.phi[c];
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < kBatch; ++q) {
-        const int b = threadIdx.x + (r0 + q) * NT;
-        if (r0 + q < kPer && b < GB) {
-          int i, j, k;
-          box_pos(b, i, j, k);
-          const int bs = i + GE * (j + GE * k);
-          styp[bs] = tv[q];
-          sphi[bs] = tv[q] >= T_OBST ? kObstacle<R>() : pv[q];
-          solid_here |= tv[q] >= T_OBST;
+    for (int q = 0; q < kBatch; ++q) {
+      const int b = threadIdx.x + (r0 + q) * NT;
+      tv[q] = 4;  // outside the domain: solid
+      pv[q] = R(0.0);
+      if (r0 + q < kPer && b < GB) {
+        int i, j, k;
+        box_pos(b, i, j, k);
+        const int X = wrapc(ox + i, p.nx, p.per[0]);
+        const int Y = wrapc(oy + j, p.ny, p.per[1]);
+        const int Z = wrapc(oz + k, p.nz, p.per[2]);
+        if (X >= 0 && Y >= 0 && Z >= 0) {
+          const int c = cidx(p, X, Y, Z);
+          tv[q] = d.flags[c] & F_TYPE;
+          if constexpr (sizeof(R) == 4) pv[q] = d.phif[c];
+          else pv[q] = d.phi[c];
         }
       }
     }
-    // without an obstacle in the box the stencils below need no
-    // substitution (most tiles)
-    const bool solid = __syncthreads_or(solid_here) != 0;
-    // The FP32 engines evaluate the same stencils grouped by z-plane.  The K8
-    // weights depend on r^2 only, so a plane contributes its centre, the sum
-    // of its 4 in-plane face neighbours and of its 4 in-plane corners; the
-    // Parker-Youngs weights (2-|d|)(2-|d'|) factor into [1 2 1] x [1 2 1] x
-    // [-1 0 1].  An obstacle point takes the value of the stencil's centre,
-    // which is the same for every plane of the window, so a plane keeps the
-    // sum over its other points and, beside it, the (weighted) count of its
-    // obstacle points, which multiplies the centre value at the end.  Each
-    // plane's sums are formed once and slide along z (other rounding than a
-    // per-cell evaluation, a fraction of its operations and registers).
-    auto planes32 = [&](auto SOLID) {
-      constexpr bool kSolid = decltype(SOLID)::value;
-      auto nz = [&](R v) { return (kSolid && is_obstacle(v)) ? R(0.0) : v; };
-      auto ob = [&](R v) { return (kSolid && is_obstacle(v)) ? R(1.0) : R(0.0); };
-      if (threadIdx.x < GS * GS) {
-        const int i = threadIdx.x % GS + 1, j = threadIdx.x / GS + 1;
-        // centre, face sum, corner sum and their obstacle counts
-        auto plane = [&](int kk, R& c0, R& f4, R& c4, R& nf, R& nc) {
-          const R* q = sphi + i + GE * (j + GE * kk);
-          c0 = q[0];
-          const R a = q[-1], b = q[1], c = q[-GE], e = q[GE];
-          const R u = q[-GE - 1], v = q[-GE + 1], w = q[GE - 1], x = q[GE + 1];
-          f4 = (nz(a) + nz(b)) + (nz(c) + nz(e));
-          c4 = (nz(u) + nz(v)) + (nz(w) + nz(x));
-          if constexpr (kSolid) {
-            nf = (ob(a) + ob(b)) + (ob(c) + ob(e));
-            nc = (ob(u) + ob(v)) + (ob(w) + ob(x));
-          }
-        };
-        R cm, fm, km, nfm = R(0.0), ncm = R(0.0);
-        R c0, f0, k0, nf0 = R(0.0), nc0 = R(0.0);
-        R cp, fp, kp, nfp = R(0.0), ncp = R(0.0);
-        plane(0, cm, fm, km, nfm, ncm);
-        plane(1, c0, f0, k0, nf0, nc0);
-        const R inv = R(1.0) / wsum;
 #pragma unroll
-        for (int k = 1; k <= GS; ++k) {
-          plane(k + 1, cp, fp, kp, nfp, ncp);
-          R out;
-          if (kSolid && is_obstacle(c0)) {
-            out = kObstacle<R>();
-          } else {
-            const R pc = c0;
-            const R zm = (kSolid && is_obstacle(cm)) ? pc : cm, zp = (kSolid && is_obstacle(cp)) ? pc : cp;
-            R s1 = (f0 + zm) + zp, s2 = (k0 + fm) + fp, s3 = km + kp;
-            if constexpr (kSolid) {
-              s1 = s1 + nf0 * pc;
-              s2 = s2 + (nc0 + nfm + nfp) * pc;
-              s3 = s3 + (ncm + ncp) * pc;
-            }
-            out = (pc + k8w<R>(1) * s1 + k8w<R>(2) * s2 + k8w<R>(3) * s3) * inv;
-          }
-          sps[(i - 1) + GS * ((j - 1) + GS * (k - 1))] = out;
-          cm = c0; fm = f0; km = k0; nfm = nf0; ncm = nc0;
-          c0 = cp; f0 = fp; k0 = kp; nf0 = nfp; nc0 = ncp;
+    for (int q = 0; q < kBatch; ++q) {
+      const int b = threadIdx.x + (r0 + q) * NT;
+      if (r0 + q < kPer && b < GB) {
+        int i, j, k;
+        box_pos(b, i, j, k);
+        const int bs = i + GE * (j + GE * k);
+        styp[bs] = tv[q];
+        sphi[bs] = tv[q] >= T_OBST ? kObstacle<R>() : pv[q];
+        solid_here |= tv[q] >= T_OBST;
+        if (tv[q] == T_IFACE && i >= 3 && i < 3 + GT && j >= 3 && j < 3 + GT && k >= 3 && k < 3 + GT &&
+            ox + i < p.nx && oy + j < p.ny && oz + k < p.nz) {
+          // an interface cell of the tile: n^ there and at its face neighbours
+          uint8_t* m = need_n + (i - 2) + GN * ((j - 2) + GN * (k - 2));
+          m[0] = 1;
+          m[-1] = 1;
+          m[1] = 1;
+          m[-GN] = 1;
+          m[GN] = 1;
+          m[-GN * GN] = 1;
+          m[GN * GN] = 1;
         }
       }
-      __syncthreads();
-      if (threadIdx.x < GN * GN) {
-        const int i = threadIdx.x % GN + 2, j = threadIdx.x / GN + 2;
-        // per plane: gx = S_y D_x psi, gy = S_x D_y psi, s = S_x S_y psi over
-        // the points that are not obstacles, and the same weights summed
-        // over the obstacle points (gxo, gyo, so)
-        auto plane = [&](int kk, R& ctr, R& gx, R& gy, R& sm, R& gxo, R& gyo, R& so) {
-          const R* q = sps + (i - 1) + GS * ((j - 1) + GS * (kk - 1));
-          const R a00 = q[-GS - 1], a01 = q[-GS], a02 = q[-GS + 1];
-          const R a10 = q[-1], a11 = q[0], a12 = q[1];
-          const R a20 = q[GS - 1], a21 = q[GS], a22 = q[GS + 1];
-          ctr = a11;
-          gx = (nz(a02) - nz(a00)) + R(2.0) * (nz(a12) - nz(a10)) + (nz(a22) - nz(a20));
-          gy = (nz(a20) - nz(a00)) + R(2.0) * (nz(a21) - nz(a01)) + (nz(a22) - nz(a02));
-          sm = (nz(a00) + R(2.0) * nz(a01) + nz(a02)) + R(2.0) * (nz(a10) + R(2.0) * nz(a11) + nz(a12)) +
-               (nz(a20) + R(2.0) * nz(a21) + nz(a22));
-          if constexpr (kSolid) {
-            gxo = (ob(a02) - ob(a00)) + R(2.0) * (ob(a12) - ob(a10)) + (ob(a22) - ob(a20));
-            gyo = (ob(a20) - ob(a00)) + R(2.0) * (ob(a21) - ob(a01)) + (ob(a22) - ob(a02));
-            so = (ob(a00) + R(2.0) * ob(a01) + ob(a02)) + R(2.0) * (ob(a10) + R(2.0) * ob(a11) + ob(a12)) +
-                 (ob(a20) + R(2.0) * ob(a21) + ob(a22));
-          }
-        };
-        R t, xm, ym, sm, xom = R(0.0), yom = R(0.0), som = R(0.0);
-        R c0, x0, y0, s0, xo0 = R(0.0), yo0 = R(0.0), so0 = R(0.0);
-        R cp, xp, yp, sp, xop = R(0.0), yop = R(0.0), sop = R(0.0);
-        plane(1, t, xm, ym, sm, xom, yom, som);
-        plane(2, c0, x0, y0, s0, xo0, yo0, so0);
-#pragma unroll
-        for (int k = 2; k < 2 + GN; ++k) {
-          plane(k + 1, cp, xp, yp, sp, xop, yop, sop);
-          R n0 = R(0.0), n1 = R(0.0), n2 = R(0.0);
-          if (!(kSolid && is_obstacle(c0))) {
-            n0 = xm + R(2.0) * x0 + xp;
-            n1 = ym + R(2.0) * y0 + yp;
-            n2 = sp - sm;
-            if constexpr (kSolid) {
-              n0 = n0 + (xom + R(2.0) * xo0 + xop) * c0;
-              n1 = n1 + (yom + R(2.0) * yo0 + yop) * c0;
-              n2 = n2 + (sop - som) * c0;
-            }
-          }
-          const R l2 = n0 * n0 + n1 * n1 + n2 * n2;
-          const R il = l2 > R(0.0) ? rsqrtf(l2) : R(0.0);
-          const int s3 = (i - 2) + GN * ((j - 2) + GN * (k - 2));
-          snh[s3] = n0 * il;
-          snh[GN * GN * GN + s3] = n1 * il;
-          snh[2 * GN * GN * GN + s3] = n2 * il;
-          xm = x0; ym = y0; sm = s0; xom = xo0; yom = yo0; som = so0;
-          c0 = cp; x0 = xp; y0 = yp; s0 = sp; xo0 = xop; yo0 = yop; so0 = sop;
-        }
-      }
-    };
-    auto stencils = [&](auto SOLID) {
-      constexpr bool kSolid = decltype(SOLID)::value;
-      // smoothed fill level on the 12^3 sub-box: one thread per z-column,
-      // the 3x3x3 window slides along z in registers
-      if (threadIdx.x < GS * GS) {
-        const int i = threadIdx.x % GS + 1, j = threadIdx.x / GS + 1;
-        R w[3][9];  // planes k-1, k, k+1 of the window, (dy, dx) row-major
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-          for (int e = 0; e < 9; ++e)
-            w[q + 1][e] = sphi[(i + e % 3 - 1) + GE * ((j + e / 3 - 1) + GE * q)];
-#pragma unroll
-        for (int k = 1; k <= GS; ++k) {
-#pragma unroll
-          for (int e = 0; e < 9; ++e) {
-            w[0][e] = w[1][e];
-            w[1][e] = w[2][e];
-            w[2][e] = sphi[(i + e % 3 - 1) + GE * ((j + e / 3 - 1) + GE * (k + 1))];
-          }
-          const R pc = w[1][4];
-          R out = kObstacle<R>();
-          if (!kSolid || !is_obstacle(pc)) {
-            R acc = R(0.0);
-#pragma unroll
-            for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-              for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-                for (int dx = -1; dx <= 1; ++dx) {
-                  const R raw = w[dz + 1][(dy + 1) * 3 + dx + 1];
-                  const R v = (kSolid && is_obstacle(raw)) ? pc : raw;
-                  acc = acc + k8w<R>(dx * dx + dy * dy + dz * dz) * v;
-                }
-            out = acc / wsum;
-          }
-          sps[(i - 1) + GS * ((j - 1) + GS * (k - 1))] = out;
-        }
-      }
-      __syncthreads();
-      // Parker-Youngs normal on the 10^3 sub-box, z-columns as above
-      if (threadIdx.x < GN * GN) {
-        const int i = threadIdx.x % GN + 2, j = threadIdx.x / GN + 2;
-        auto psi = [&](int ii, int jj, int kk) { return sps[(ii - 1) + GS * ((jj - 1) + GS * (kk - 1))]; };
-        R w[3][9];
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-          for (int e = 0; e < 9; ++e) w[q + 1][e] = psi(i + e % 3 - 1, j + e / 3 - 1, 1 + q);
-#pragma unroll
-        for (int k = 2; k < 2 + GN; ++k) {
-#pragma unroll
-          for (int e = 0; e < 9; ++e) {
-            w[0][e] = w[1][e];
-            w[1][e] = w[2][e];
-            w[2][e] = psi(i + e % 3 - 1, j + e / 3 - 1, k + 1);
-          }
-          auto at = [&](int dx, int dy, int dz) { return w[dz + 1][(dy + 1) * 3 + dx + 1]; };
-          const R pc = at(0, 0, 0);
-          R out[3] = {R(0.0), R(0.0), R(0.0)};
-          if (!kSolid || !is_obstacle(pc)) {
-            R nn[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-              R acc = R(0.0);
-#pragma unroll
-              for (int pp = -1; pp <= 1; ++pp)
-#pragma unroll
-                for (int r = -1; r <= 1; ++r) {
-                  const int ax = (a == 0) ? 1 : r, ay = (a == 0) ? r : (a == 1) ? 1 : pp,
-                            az = (a == 2) ? 1 : pp;
-                  const int bx = (a == 0) ? -1 : ax, by = (a == 1) ? -1 : ay, bz = (a == 2) ? -1 : az;
-                  const R rp = at(ax, ay, az), rm = at(bx, by, bz);
-                  const R vp = (kSolid && is_obstacle(rp)) ? pc : rp;
-                  const R vm = (kSolid && is_obstacle(rm)) ? pc : rm;
-                  const R wt = (pp == 0 && r == 0) ? R(4.0) : (pp == 0 || r == 0) ? R(2.0) : R(1.0);
-                  acc = acc + wt * (vp - vm);
-                }
-              nn[a] = acc;
-            }
-            const R len = sqrt(nn[0] * nn[0] + nn[1] * nn[1] + nn[2] * nn[2]);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) out[a] = (len > R(0.0)) ? nn[a] / len : R(0.0);
-          }
-          const int s3 = (i - 2) + GN * ((j - 2) + GN * (k - 2));
-          snh[s3] = out[0];
-          snh[GN * GN * GN + s3] = out[1];
-          snh[2 * GN * GN * GN + s3] = out[2];
-        }
-      }
-    };
-    if constexpr (sizeof(R) == 4) {
-      if (solid) planes32(std::true_type{});
-      else planes32(std::false_type{});
-    } else {
-      if (solid) stencils(std::true_type{});
-      else stencils(std::false_type{});
     }
-    __syncthreads();
-    // curvature, gas density and Thuerey class of the tile's interface cells
-    for (int s = threadIdx.x; s < GT * GT * GT; s += blockDim.x) {
-      const int i = s % GT + 3, j = (s / GT) % GT + 3, k = s / (GT * GT) + 3;
-      const int X = ox + i, Y = oy + j, Z = oz + k;
-      if (X >= p.nx || Y >= p.ny || Z >= p.nz) continue;
-      const int b = i + GE * (j + GE * k);
-      if (styp[b] != T_IFACE) continue;
-      const int c = cidx(p, X, Y, Z);
-      auto nh = [&](int a, int ii, int jj, int kk) {
-        return snh[a * GN * GN * GN + (ii - 2) + GN * ((jj - 2) + GN * (kk - 2))];
-      };
-      R acc = R(0.0);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const int ex = (a == 0), ey = (a == 1), ez = (a == 2);
-        const R vc = nh(a, i, j, k);
-        const R vp = (styp[b + ex + GE * (ey + GE * ez)] >= T_OBST) ? vc : nh(a, i + ex, j + ey, k + ez);
-        const R vm = (styp[b - ex - GE * (ey + GE * ez)] >= T_OBST) ? vc : nh(a, i - ex, j - ey, k - ez);
-        acc = acc + (vp - vm);
-      }
-      const R kappa = R(-0.5) * acc;
-      const int bb = d.bid[c];
-      if constexpr (S::kDev) {
-        // rho^G - 1 = 3 (p^V - 1/3) + 3 sigma kappa, formed in FP64
-        const double pv = (p.bubble_model && bb >= 0) ? d.pV[bb] : p.pv0;
-        rhog[c] = R(3.0 * (pv - 1.0 / 3.0) + 3.0 * p.sigma * (double)kappa);
-      } else {
-        const R pv = (p.bubble_model && bb >= 0) ? R(d.pV[bb]) : R(p.pv0);
-        rhog[c] = R(3.0) * (pv + R(p.sigma) * kappa);
-      }
-      nhat[3LL * c + 0] = nh(0, i, j, k);
-      nhat[3LL * c + 1] = nh(1, i, j, k);
-      nhat[3LL * c + 2] = nh(2, i, j, k);
-      bool hl = false, hg = false;
-#pragma unroll
-      for (int q = 1; q < Q; ++q) {
-        const int t = styp[b + CX(q) + GE * (CY(q) + GE * CZ(q))];
-        hl |= (t == T_LIQ);
-        hg |= (t == T_GAS);
-      }
-      d.cls[c] = T_IFACE | (((!hl && hg) ? CL_NF : (hl && !hg) ? CL_NE : CL_STD) << 2);
-    }
-    if (threadIdx.x == 0) d.tile_mark[tile] = 0;
   }
+  // without an obstacle in the box the stencils below need no substitution
+  // (most tiles)
+  const bool solid = __syncthreads_or(solid_here) != 0;
+  for (int base = 0; base < GN3; base += NT) {
+    const int s = base + threadIdx.x;
+    bool take = false;
+    int ss = 0;
+    if (s < GN3 && need_n[s]) {
+      const int i = s % GN + 2, j = (s / GN) % GN + 2, k = s / (GN * GN) + 2;
+      take = styp[i + GE * (j + GE * k)] < T_OBST;  // at an obstacle the centre's n^ stands in
+      ss = (i - 1) + GS * ((j - 1) + GS * (k - 1));
+    }
+    if (take) {
+#pragma unroll
+      for (int e = 0; e < 27; ++e) need_s[ss + (e % 3 - 1) + GS * (((e / 3) % 3 - 1) + GS * (e / 9 - 1))] = 1;
+    }
+    push_shared(list_n, &s_count[0], take, s);
+  }
+  __syncthreads();
+  for (int base = 0; base < GS3; base += NT) {
+    const int s = base + threadIdx.x;
+    push_shared(list_s, &s_count[1], s < GS3 && need_s[s], s);
+  }
+  __syncthreads();
+  auto smooth = [&](auto SOLID) {
+    constexpr bool kSolid = decltype(SOLID)::value;
+    const int n = s_count[1];
+    for (int q = threadIdx.x; q < n; q += NT) {
+      const int s = list_s[q];
+      const int b = (s % GS + 1) + GE * ((s / GS) % GS + 1 + GE * (s / (GS * GS) + 1));
+      sps[s] = (kSolid && is_obstacle(sphi[b])) ? kObstacle<R>() : smoothed_at<R, kSolid>(sphi, b);
+    }
+  };
+  if (solid) smooth(std::true_type{});
+  else smooth(std::false_type{});
+  __syncthreads();
+  auto normals = [&](auto SOLID) {
+    constexpr bool kSolid = decltype(SOLID)::value;
+    const int n = s_count[0];
+    for (int q = threadIdx.x; q < n; q += NT) {
+      const int s = list_n[q];
+      R v[3];
+      normal_at<R, kSolid>(sps, (s % GN + 1) + GS * ((s / GN) % GN + 1 + GS * (s / (GN * GN) + 1)), v);
+      snh[s] = v[0];
+      snh[GN3 + s] = v[1];
+      snh[2 * GN3 + s] = v[2];
+    }
+  };
+  if (solid) normals(std::true_type{});
+  else normals(std::false_type{});
+  __syncthreads();
+  // curvature, gas density and Thuerey class of the tile's interface cells
+  for (int s = threadIdx.x; s < GT * GT * GT; s += blockDim.x) {
+    const int i = s % GT + 3, j = (s / GT) % GT + 3, k = s / (GT * GT) + 3;
+    const int X = ox + i, Y = oy + j, Z = oz + k;
+    if (X >= p.nx || Y >= p.ny || Z >= p.nz) continue;
+    const int b = i + GE * (j + GE * k);
+    if (styp[b] != T_IFACE) continue;
+    const int c = cidx(p, X, Y, Z);
+    auto nh = [&](int a, int ii, int jj, int kk) {
+      return snh[a * GN3 + (ii - 2) + GN * ((jj - 2) + GN * (kk - 2))];
+    };
+    R acc = R(0.0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const int ex = (a == 0), ey = (a == 1), ez = (a == 2);
+      const R vc = nh(a, i, j, k);
+      const R vp = (styp[b + ex + GE * (ey + GE * ez)] >= T_OBST) ? vc : nh(a, i + ex, j + ey, k + ez);
+      const R vm = (styp[b - ex - GE * (ey + GE * ez)] >= T_OBST) ? vc : nh(a, i - ex, j - ey, k - ez);
+      acc = acc + (vp - vm);
+    }
+    const R kappa = R(-0.5) * acc;
+    const int bb = d.bid[c];
+    if constexpr (S::kDev) {
+      // rho^G - 1 = 3 (p^V - 1/3) + 3 sigma kappa, formed in FP64
+      const double pv = (p.bubble_model && bb >= 0) ? d.pV[bb] : p.pv0;
+      rhog[c] = R(3.0 * (pv - 1.0 / 3.0) + 3.0 * p.sigma * (double)kappa);
+    } else {
+      const R pv = (p.bubble_model && bb >= 0) ? R(d.pV[bb]) : R(p.pv0);
+      rhog[c] = R(3.0) * (pv + R(p.sigma) * kappa);
+    }
+    nhat[3LL * c + 0] = nh(0, i, j, k);
+    nhat[3LL * c + 1] = nh(1, i, j, k);
+    nhat[3LL * c + 2] = nh(2, i, j, k);
+    bool hl = false, hg = false;
+#pragma unroll
+    for (int q = 1; q < Q; ++q) {
+      const int t = styp[b + CX(q) + GE * (CY(q) + GE * CZ(q))];
+      hl |= (t == T_LIQ);
+      hg |= (t == T_GAS);
+    }
+    d.cls[c] = T_IFACE | (((!hl && hg) ? CL_NF : (hl && !hg) ? CL_NE : CL_STD) << 2);
+  }
+  if (threadIdx.x == 0) d.tile_mark[tile] = 0;
+}
 
 // Resets the work-list counters that this step fills (next band list, new
 // cells, next tile list, converting cells, receivers).
