@@ -393,10 +393,6 @@ constexpr int GB = GE * GE * GE;         // 2744 box positions
 constexpr int GS = GT + 4;               // phi~ sub-box edge (12)
 constexpr int GN = GT + 2;               // n^ sub-box edge (10)
 constexpr int kGeoBlock = 256;
-#ifndef FSLBM_GEO_LOAD_BATCH
-#define FSLBM_GEO_LOAD_BATCH 6
-#endif
-constexpr int kGeoLoadBatch = FSLBM_GEO_LOAD_BATCH;  // box positions a thread loads at once
 // geometry blocks per interface-band block: each tile's block runs four
 // dependent shared-memory phases, so many resident tiles hide the latency
 #ifndef FSLBM_GEO_MULT
@@ -438,15 +434,30 @@ __device__ __forceinline__ double div_k8(double a) {
   return fma(a, 0x1.1648d50fc3201p-2, a * 0x1.648d50fc32011p-58);
 }
 
-// Warp-wide append to a list in shared memory; every lane calls it.
-__device__ __forceinline__ void push_shared(unsigned short* list, int* count, bool take, int value) {
-  const unsigned m = __ballot_sync(0xffffffffu, take);
-  if (!m) return;
+// Appends the positions s = t, t + NT, ... < n of thread t that have bit r of
+// take set (r-th position) to a list in shared memory, one atomic a warp;
+// every lane calls it.
+template <int N, int NT>
+__device__ __forceinline__ void push_shared(unsigned short* list, int* count, unsigned take) {
+  constexpr int kPer = (N + NT - 1) / NT;
   const unsigned lane = threadIdx.x & 31u;
+  unsigned m[kPer];
+  int total = 0;
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    m[r] = __ballot_sync(0xffffffffu, (take >> r) & 1u);
+    total += __popc(m[r]);
+  }
+  if (total == 0) return;
   int base = 0;
-  if (lane == 0) base = atomicAdd(count, __popc(m));
+  if (lane == 0) base = atomicAdd(count, total);
   base = __shfl_sync(0xffffffffu, base, 0);
-  if (take) list[base + __popc(m & ((1u << lane) - 1u))] = (unsigned short)value;
+#pragma unroll
+  for (int r = 0; r < kPer; ++r) {
+    if ((take >> r) & 1u)
+      list[base + __popc(m[r] & ((1u << lane) - 1u))] = (unsigned short)(threadIdx.x + r * NT);
+    base += __popc(m[r]);
+  }
 }
 
 // phi~ at box position b (not an obstacle).  The FP32 engines group the 27
@@ -579,8 +590,8 @@ template <int Q, class S, int NT = kGeoBlock>
 __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, int tile,
                                               unsigned char* g_smem) {
   using R = typename S::Real;
-  constexpr int kPer = (GB + NT - 1) / NT;  // box positions per thread
-  __shared__ int s_count[2];                // points in the lists
+  __shared__ int s_count[2];      // points in the lists
+  __shared__ int s_off[3][16];    // offsets of the box coordinates
   R* sphi = (R*)g_smem;
   R* snh = sphi;  // written after the smoothing's last read of sphi
   R* sps = sphi + kGeoBoxSlots;
@@ -598,59 +609,70 @@ __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, 
   __syncthreads();  // the previous tile is done with the buffers
   for (int w = threadIdx.x; w < (GN3 + GS3) / 4; w += NT) ((unsigned*)need_n)[w] = 0u;
   if (threadIdx.x < 2) s_count[threadIdx.x] = 0;
+  if (threadIdx.x < 48) {
+    // offset of box position k along storage axis a, -1 outside the domain
+    // (and outside the box)
+    const int a = threadIdx.x >> 4, k = threadIdx.x & 15, x = p.ax[a];
+    const int X = wrapc(sel3(x, ox, oy, oz) + k, sel3(x, p.nx, p.ny, p.nz), sel3(x, p.per[0], p.per[1], p.per[2]));
+    s_off[a][k] = X < 0 || k >= GE ? -1 : X * sel3(x, p.sx, p.sy, p.sz);
+  }
   __syncthreads();
-  // Thread t loads box position t + r NT counted in the cells' storage order
-  // (its first coordinate runs along the contiguous axis), so that the loads
-  // of a warp coalesce whatever the storage order; the shared-memory box
+  // The box in the cells' storage order: 16 lanes take the 14 positions of a
+  // row along the contiguous axis (the loads of a warp coalesce whatever the
+  // storage order), the threads' rows advance by NT / 16.  The offsets of the
+  // coordinates along each axis come from a table.  All of a thread's global
+  // reads are issued before the first result is used, without a branch around
+  // them (positions outside read cell 0): a branch a position made the thread
+  // wait for every load in turn, 6 to 7 us a tile.  The shared-memory box
   // itself is indexed in the caller's axes.
-  auto box_pos = [&](int b, int& i, int& j, int& k) {
-    const int k0 = b % GE, k1 = (b / GE) % GE, k2 = b / (GE * GE);
-    i = sel3(p.inv[0], k0, k1, k2);
-    j = sel3(p.inv[1], k0, k1, k2);
-    k = sel3(p.inv[2], k0, k1, k2);
-  };
-  // in rounds of at most kBatch positions, all of whose global reads are
-  // issued before the first shared-memory store (the loads in flight fit the
-  // registers of a 64-register thread)
-  constexpr int kBatch = kGeoLoadBatch < kPer ? kGeoLoadBatch : kPer;
+  constexpr int kRowStep = NT / 16;
+  constexpr int kRows = (GE * GE + kRowStep - 1) / kRowStep;  // rows per thread
+  static_assert(NT % 16 == 0 && kRowStep >= GE && kRowStep < 2 * GE, "row walk");
+  const int o[3] = {ox, oy, oz}, size[3] = {p.nx, p.ny, p.nz};
+  const int k0 = threadIdx.x & 15;
+  // steps of the storage axes in the shared-memory box (caller's axes)
+  int bstep[3], core[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int x = p.ax[a];
+    bstep[a] = x == 0 ? 1 : x == 1 ? GE : GE * GE;
+    const int left = sel3(x, size[0] - o[0], size[1] - o[1], size[2] - o[2]) - 3;
+    core[a] = left < GT ? left : GT;  // the tile's cells inside the domain
+  }
   bool solid_here = false;  // an obstacle or a position outside the domain
+  {
+    uint8_t tv[kRows];
+    R pv[kRows];
+    unsigned inside = 0u;  // bit r: position r lies in the domain
+    int k1 = threadIdx.x >> 4, k2 = 0;
+    if (k1 >= GE) k1 -= GE, k2 = 1;
 #pragma unroll
-  for (int r0 = 0; r0 < kPer; r0 += kBatch) {
-    uint8_t tv[kBatch];
-    R pv[kBatch];
-#pragma unroll
-    for (int q = 0; q < kBatch; ++q) {
-      const int b = threadIdx.x + (r0 + q) * NT;
-      tv[q] = 4;  // outside the domain: solid
-      pv[q] = R(0.0);
-      if (r0 + q < kPer && b < GB) {
-        int i, j, k;
-        box_pos(b, i, j, k);
-        const int X = wrapc(ox + i, p.nx, p.per[0]);
-        const int Y = wrapc(oy + j, p.ny, p.per[1]);
-        const int Z = wrapc(oz + k, p.nz, p.per[2]);
-        if (X >= 0 && Y >= 0 && Z >= 0) {
-          const int c = cidx(p, X, Y, Z);
-          tv[q] = d.flags[c] & F_TYPE;
-          if constexpr (sizeof(R) == 4) pv[q] = d.phif[c];
-          else pv[q] = d.phi[c];
-        }
-      }
+    for (int r = 0; r < kRows; ++r) {
+      const int e0 = s_off[0][k0], e1 = s_off[1][k1], e2 = s_off[2][k2];
+      const bool in = (e0 | e1 | e2) >= 0;
+      inside |= (unsigned)in << r;
+      const int c = in ? e0 + e1 + e2 : 0;
+      tv[r] = d.flags[c];
+      if constexpr (sizeof(R) == 4) pv[r] = d.phif[c];
+      else pv[r] = d.phi[c];
+      k1 += kRowStep - GE, k2 += 1;
+      if (k1 >= GE) k1 -= GE, k2 += 1;
     }
+    k1 = threadIdx.x >> 4, k2 = 0;
+    if (k1 >= GE) k1 -= GE, k2 = 1;
 #pragma unroll
-    for (int q = 0; q < kBatch; ++q) {
-      const int b = threadIdx.x + (r0 + q) * NT;
-      if (r0 + q < kPer && b < GB) {
-        int i, j, k;
-        box_pos(b, i, j, k);
-        const int bs = i + GE * (j + GE * k);
-        styp[bs] = tv[q];
-        sphi[bs] = tv[q] >= T_OBST ? kObstacle<R>() : pv[q];
-        solid_here |= tv[q] >= T_OBST;
-        if (tv[q] == T_IFACE && i >= 3 && i < 3 + GT && j >= 3 && j < 3 + GT && k >= 3 && k < 3 + GT &&
-            ox + i < p.nx && oy + j < p.ny && oz + k < p.nz) {
+    for (int r = 0; r < kRows; ++r) {
+      if (k0 < GE && k2 < GE) {
+        const int bs = k0 * bstep[0] + k1 * bstep[1] + k2 * bstep[2];
+        const uint8_t t = ((inside >> r) & 1u) ? (uint8_t)(tv[r] & F_TYPE) : (uint8_t)4;  // outside: solid
+        styp[bs] = t;
+        sphi[bs] = t >= T_OBST ? kObstacle<R>() : pv[r];
+        solid_here |= t >= T_OBST;
+        if (t == T_IFACE && (unsigned)(k0 - 3) < (unsigned)core[0] && (unsigned)(k1 - 3) < (unsigned)core[1] &&
+            (unsigned)(k2 - 3) < (unsigned)core[2]) {
           // an interface cell of the tile: n^ there and at its face neighbours
-          uint8_t* m = need_n + (i - 2) + GN * ((j - 2) + GN * (k - 2));
+          uint8_t* m = need_n + (sel3(p.inv[0], k0, k1, k2) - 2) +
+                       GN * ((sel3(p.inv[1], k0, k1, k2) - 2) + GN * (sel3(p.inv[2], k0, k1, k2) - 2));
           m[0] = 1;
           m[-1] = 1;
           m[1] = 1;
@@ -660,31 +682,36 @@ __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, 
           m[GN * GN] = 1;
         }
       }
+      k1 += kRowStep - GE, k2 += 1;
+      if (k1 >= GE) k1 -= GE, k2 += 1;
     }
   }
   // without an obstacle in the box the stencils below need no substitution
   // (most tiles)
   const bool solid = __syncthreads_or(solid_here) != 0;
-  for (int base = 0; base < GN3; base += NT) {
-    const int s = base + threadIdx.x;
-    bool take = false;
-    int ss = 0;
+  unsigned take = 0u;
+#pragma unroll
+  for (int r = 0; r < (GN3 + NT - 1) / NT; ++r) {
+    const int s = threadIdx.x + r * NT;
     if (s < GN3 && need_n[s]) {
       const int i = s % GN + 2, j = (s / GN) % GN + 2, k = s / (GN * GN) + 2;
-      take = styp[i + GE * (j + GE * k)] < T_OBST;  // at an obstacle the centre's n^ stands in
-      ss = (i - 1) + GS * ((j - 1) + GS * (k - 1));
-    }
-    if (take) {
+      if (styp[i + GE * (j + GE * k)] < T_OBST) {  // at an obstacle the centre's n^ stands in
+        take |= 1u << r;
+        uint8_t* m = need_s + (i - 1) + GS * ((j - 1) + GS * (k - 1));
 #pragma unroll
-      for (int e = 0; e < 27; ++e) need_s[ss + (e % 3 - 1) + GS * (((e / 3) % 3 - 1) + GS * (e / 9 - 1))] = 1;
+        for (int e = 0; e < 27; ++e) m[(e % 3 - 1) + GS * (((e / 3) % 3 - 1) + GS * (e / 9 - 1))] = 1;
+      }
     }
-    push_shared(list_n, &s_count[0], take, s);
   }
+  push_shared<GN3, NT>(list_n, &s_count[0], take);
   __syncthreads();
-  for (int base = 0; base < GS3; base += NT) {
-    const int s = base + threadIdx.x;
-    push_shared(list_s, &s_count[1], s < GS3 && need_s[s], s);
+  take = 0u;
+#pragma unroll
+  for (int r = 0; r < (GS3 + NT - 1) / NT; ++r) {
+    const int s = threadIdx.x + r * NT;
+    take |= (unsigned)(s < GS3 && need_s[s]) << r;
   }
+  push_shared<GS3, NT>(list_s, &s_count[1], take);
   __syncthreads();
   auto smooth = [&](auto SOLID) {
     constexpr bool kSolid = decltype(SOLID)::value;
@@ -734,13 +761,13 @@ __device__ __forceinline__ void geometry_tile(const DPtrs& d, const KParams& p, 
       acc = acc + (vp - vm);
     }
     const R kappa = R(-0.5) * acc;
-    const int bb = d.bid[c];
+    const int bb = p.bubble_model ? d.bid[c] : -1;
     if constexpr (S::kDev) {
       // rho^G - 1 = 3 (p^V - 1/3) + 3 sigma kappa, formed in FP64
-      const double pv = (p.bubble_model && bb >= 0) ? d.pV[bb] : p.pv0;
+      const double pv = bb >= 0 ? d.pV[bb] : p.pv0;
       rhog[c] = R(3.0 * (pv - 1.0 / 3.0) + 3.0 * p.sigma * (double)kappa);
     } else {
-      const R pv = (p.bubble_model && bb >= 0) ? R(d.pV[bb]) : R(p.pv0);
+      const R pv = bb >= 0 ? R(d.pV[bb]) : R(p.pv0);
       rhog[c] = R(3.0) * (pv + R(p.sigma) * kappa);
     }
     nhat[3LL * c + 0] = nh(0, i, j, k);
@@ -777,39 +804,41 @@ __global__ void __launch_bounds__(kGeoBlock, kGeoMinBlocks) k_geometry(DPtrs d, 
     geometry_tile<Q, S>(d, p, d.tiles[parity][tt], g_smem);
 }
 
-// The bulk sweep with the geometry pass folded in (FP32 and 16-bit
-// engines).  Every kGeoFuseEvery-th block of the persistent grid first
-// takes geometry tiles, one at a time from a per-step counter (counts[7]:
-// zero at init, cleared again by the finalize kernel of every step), until
-// none is left, and then joins the other blocks on the bulk units.  The
-// tiles so run at the sweep's occupancy (four blocks of 256 threads per SM
-// instead of three of 192) with no launch boundary before the sweep.  On the
-// 160x160x1024 Taylor bubble: separate kernels 77.5 + 295 us, every block
-// first on tiles (1) 345 us, every second block (2) 364 us, every fourth
-// 361 us: the sweep needs all its blocks to keep HBM busy, so blocks held
-// by tiles slow it by about what running the tiles beside it saves.
-#ifndef FSLBM_GEO_FUSE_EVERY
-#define FSLBM_GEO_FUSE_EVERY 1
-#endif
-constexpr int kGeoFuseEvery = FSLBM_GEO_FUSE_EVERY;
+// Hand-out of n geometry tiles to the blocks of a persistent grid: block b
+// takes tile b, later ones come from a per-step counter (zero at init, cleared
+// again every step).  Blocks without a tile go on at once, and with at most a
+// tile a block nothing waits for the counter (608 atomics on one address and
+// two barriers took 2 us of every block).
+template <class F>
+__device__ __forceinline__ void hand_out_tiles(int n, int* counter, int* s_tile, F tile) {
+  int t = blockIdx.x;
+  while (t < n) {
+    tile(t);
+    if (n <= (int)gridDim.x) break;
+    __syncthreads();  // every thread has read the previous *s_tile
+    if (threadIdx.x == 0) *s_tile = gridDim.x + atomicAdd(counter, 1);
+    __syncthreads();
+    t = *s_tile;
+  }
+}
 
+// The bulk sweep with the geometry pass folded in (FP32 and 16-bit
+// engines).  The blocks of the persistent grid first take geometry tiles
+// until none is left, and then bulk units.  The tiles so run at the sweep's
+// occupancy with no launch boundary before the sweep.  On the 160x160x1024
+// Taylor bubble: separate kernels 77.5 + 295 us, every block first on tiles
+// 345 us, every second block 364 us, every fourth 361 us: the sweep needs all
+// its blocks to keep HBM busy, so blocks held by tiles slow it by about what
+// running the tiles beside it saves.
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     k_bulk_geo(DPtrs d, KParams p, int parity) {
   extern __shared__ __align__(16) unsigned char g_smem[];
   __shared__ int s_tile;
   if (blockIdx.x == 0 && threadIdx.x == 0) reset_step_counts(d, parity);
-  if (blockIdx.x % kGeoFuseEvery == 0) {
-    const int ntiles = d.counts[3 + parity];
-    for (;;) {
-      __syncthreads();  // every thread has read the previous s_tile
-      if (threadIdx.x == 0) s_tile = atomicAdd(&d.counts[7], 1);
-      __syncthreads();
-      const int tt = s_tile;
-      if (tt >= ntiles) break;
-      geometry_tile<Q, S, kBulkBlock>(d, p, d.tiles[parity][tt], g_smem);
-    }
-  }
+  hand_out_tiles(d.counts[3 + parity], &d.counts[7], &s_tile, [&](int t) {
+    geometry_tile<Q, S, kBulkBlock>(d, p, d.tiles[parity][t], g_smem);
+  });
   bulk_sweep<Q, S, COLL>(d, p, parity);
 }
 
@@ -1550,25 +1579,17 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     kb_bulk_geo(const DomRec* __restrict__ recs, BatchPlan pl) {
   extern __shared__ __align__(16) unsigned char g_smem[];
   __shared__ int s_tile;
-  if (blockIdx.x % kGeoFuseEvery == 0) {
-    const int total = pl.tiles[pl.n];
-    for (;;) {
-      __syncthreads();  // every thread has read the previous s_tile
-      if (threadIdx.x == 0) s_tile = atomicAdd(&pl.ctr[1], 1);
-      __syncthreads();
-      const int t = s_tile;
-      if (t >= total) break;
-      const int k = find_domain(pl.tiles, pl.n, t);
-      const DomRec& r = recs[k];
-      geometry_tile<Q, S, kBulkBlock>(r.d, r.p, r.d.tiles[r.parity][t - pl.tiles[k]], g_smem);
-    }
-  }
+  hand_out_tiles(pl.tiles[pl.n], &pl.ctr[1], &s_tile, [&](int t) {
+    const int k = find_domain(pl.tiles, pl.n, t);
+    const DomRec& r = recs[k];
+    geometry_tile<Q, S, kBulkBlock>(r.d, r.p, r.d.tiles[r.parity][t - pl.tiles[k]], g_smem);
+  });
   batch_bulk_sweep<Q, S, COLL>(recs, pl);
 }
 
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) kb_interface(const DomRec* __restrict__ recs, BatchPlan pl) {
-  const int total = pl.band[pl.n];
+  const int total = pl.band[pl.n];  // with each domain's cells rounded up to whole warps
   for (int g = band_start(total); g < total; g += gridDim.x * blockDim.x) {
     const int k = find_domain(pl.band, pl.n, g);
     const DomRec& r = recs[k];
