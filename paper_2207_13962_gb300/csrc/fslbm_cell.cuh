@@ -604,6 +604,21 @@ __device__ __forceinline__ void post_moments(const typename S::T* P, long long N
   u[2] = jz / rr - R(0.5) * gpar<R>(p, 2);
 }
 
+// load_w and load_own for a run-time direction with weight w.
+template <class S>
+__device__ __forceinline__ typename S::Real load_lane(typename S::T v, typename S::Real w) {
+  if constexpr (S::kDev) return S::loadd(v);
+  else return S::load(v, w);
+}
+template <int Q, class S>
+__device__ __forceinline__ typename S::Real load_own_lane(const typename S::T* P, long long Np, long long c, int i,
+                                                          typename S::Real w) {
+  if constexpr (S::kExactRest) {
+    if (i == 0) return from_steps<S>(rest_slice<Q, S>(P, Np)[c]);
+  }
+  return load_lane<S>(P[(long long)i * Np + c], w);
+}
+
 // ------------------------------------------------- bounce-back via obstacle slots
 // Pull source of direction i of the cell at (x, y, z) (Eq. nm-lbm-streaming):
 // the cell x - c_i, wrapped across periodic faces, whose PDF i arrives

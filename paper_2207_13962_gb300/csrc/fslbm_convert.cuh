@@ -434,8 +434,8 @@ __device__ __forceinline__ void apply_old_items(const DPtrs& d, const KParams& p
 
 // The kinds of cells are disjoint and read only what earlier kernels wrote:
 // in one launch, or as two side by side in the step's graph (kNew, kOld:
-// which parts a launch does), where the stage takes the longer chain, the
-// new cells'.
+// which parts a launch does).  In one launch the new cells (the longest
+// chains) are dealt from the first warp, the others from the last.
 template <int Q, class S, bool kNew, bool kOld>
 __global__ void __launch_bounds__(kBlock) k_apply(DPtrs d, KParams p, int parity) {
   const LaneDir l = lane_dir<Q>();

@@ -276,14 +276,14 @@ struct Engine {
       o.bulk_fn[7] = (const void*)&k_bulk<Q, S, 7>;
     }
     o.bulk_blocks_per_sm = bulk_blocks_per_sm();
-    // bulk and geometry (one launch when fused), interface, resolve, count,
-    // apply (two launches when fused), finalize, list rebuild
+    // bulk and geometry (one launch when fused), interface, resolve,
+    // count, apply (two launches when fused), finalize, list rebuild
     o.step_launches = 8;
     o.bulk_smem = kTmaBulk ? tma_smem<Q, typename S::T>() : kFusedGeo ? geometry_smem<typename S::Real>() : 0;
     o.batch_step = &batch_step;
-    // plan, geometry, bulk sweep (one launch when fused), interface update,
-    // resolve, count, apply (two in FP64), finalize, bubbles + buffer swap,
-    // and kb_compact_band, launched by the batch
+    // plan, geometry and bulk sweep (one launch when fused), interface update,
+    // resolve, count, apply (two in FP64), finalize,
+    // bubbles + buffer swap, and kb_compact_band, launched by the batch
     o.batch_step_launches = kFusedGeo ? 9 : 11;
     if constexpr (kFusedGeo) {
       const void* fns[8] = {(const void*)&kb_bulk_geo<Q, S, 0>, (const void*)&kb_bulk_geo<Q, S, 1>,

@@ -26,6 +26,7 @@
 
 #include "fslbm_bulk_tma.cuh"
 #include "fslbm_convert.cuh"
+#include "fslbm_interface_lanes.cuh"
 #include <type_traits>
 
 namespace fslbm {
@@ -1141,8 +1142,12 @@ __device__ __forceinline__ int band_start(int n) {
 }
 
 template <int Q, class S, int COLL>
-__global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) k_interface(DPtrs d, KParams p, int parity) {
+__global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) k_interface(const __grid_constant__ DPtrs d, const __grid_constant__ KParams p, int parity) {
   const int n = d.counts[parity];
+  if (lane_band<Q, S>(n)) {
+    interface_by_lanes<Q, S, COLL>(d, p, parity, n);
+    return;
+  }
   bool bad = false;
   for (int k = band_start(n); k < n; k += gridDim.x * blockDim.x)
     interface_cell<Q, S, COLL>(d, p, parity, k, bad);
@@ -1590,6 +1595,10 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) kb_interface(const DomRec* __restrict__ recs, BatchPlan pl) {
   const int total = pl.band[pl.n];  // with each domain's cells rounded up to whole warps
+  if (lane_band<Q, S>(total)) {
+    interface_by_lanes<Q, S, COLL>(recs, pl.band, pl.n, total);
+    return;
+  }
   for (int g = band_start(total); g < total; g += gridDim.x * blockDim.x) {
     const int k = find_domain(pl.band, pl.n, g);
     const DomRec& r = recs[k];
