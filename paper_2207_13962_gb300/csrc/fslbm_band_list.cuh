@@ -72,19 +72,29 @@ __device__ __forceinline__ void compact_chunk(const uint8_t* __restrict__ flags,
   __syncthreads();  // s_warp and s_base are rewritten by the next chunk
 }
 
-// Single domain, after k_finalize (which leaves the next list empty).
-static __global__ void __launch_bounds__(kBlock) k_compact_band(DPtrs d, KParams p, int parity) {
-  const long long N = p.N;
-  for (long long chunk = (long long)blockIdx.x * kCompactChunk; chunk < N;
-       chunk += (long long)gridDim.x * kCompactChunk)
+// Single domain, after k_finalize (which leaves the next list empty and the
+// bubbles' volume sums complete).  The first bubble_blocks (0 or 1) blocks
+// update the bubble pressures, which need nothing of the list; the others
+// take the chunks.
+static __global__ void __launch_bounds__(kBlock) k_compact_band(DPtrs d, KParams p, int parity, int bubble_blocks) {
+  stage_begin();
+  const int block = (int)blockIdx.x - bubble_blocks;
+  if (block < 0) {
+    bubble_update(d, p);
+    return;
+  }
+  const long long N = p.N, blocks = (int)gridDim.x - bubble_blocks;
+  for (long long chunk = block * (long long)kCompactChunk; chunk < N; chunk += blocks * kCompactChunk)
     compact_chunk(d.flags, N, chunk, d.band[parity ^ 1], &d.counts[parity ^ 1]);
 }
 
 // All domains of a batch, at the end of a batched step (after the buffer
 // swap, so a domain's next list is band[parity]).  chunk_off[k]: prefix of
-// the domains' chunk counts (n + 1 entries).
-static __global__ void __launch_bounds__(kBlock) kb_compact_band(const DomRec* __restrict__ recs,
-                                                                 const int* __restrict__ chunk_off, int n) {
+// the domains' chunk counts (n + 1 entries).  recs is not __restrict__: the
+// kernel before writes the parities, which must not be read before the wait.
+static __global__ void __launch_bounds__(kBlock) kb_compact_band(const DomRec* recs, const int* __restrict__ chunk_off,
+                                                                 int n) {
+  stage_begin();
   const int total = chunk_off[n];
   for (int g = blockIdx.x; g < total; g += gridDim.x) {
     const int k = find_domain(chunk_off, n, g);

@@ -63,8 +63,8 @@ cudaError_t capture(fslbm_batch* b) {
   b->ops.batch_step(b->d_recs, b->plan, b->sms * b->tune.band_blocks_per_sm,
                     b->sms * b->tune.bulk_blocks_per_sm, b->collision, b->cap, &b->fork);
   // every member's next interface list in cell order
-  kb_compact_band<<<b->nchunks < 8 * b->sms ? b->nchunks : 8 * b->sms, kBlock, 0, b->cap>>>(
-      b->d_recs, b->d_chunk, (int)b->m.size());
+  launch_stage(true, kb_compact_band, b->nchunks < 8 * b->sms ? b->nchunks : 8 * b->sms, kBlock, 0, b->cap,
+               b->d_recs, b->d_chunk, (int)b->m.size());
   e = cudaStreamEndCapture(b->cap, &g);
   if (e != cudaSuccess) return e;
   e = prioritise_nodes(g, b->ops.batch_bulk_fn[b->collision], nullptr);

@@ -167,6 +167,7 @@ __device__ __forceinline__ void bulk_sweep(const DPtrs& d, const KParams& p, int
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     k_bulk(DPtrs d, KParams p, int parity) {
+  stage_begin();
   bulk_sweep<Q, S, COLL>(d, p, parity);
 }
 

@@ -398,6 +398,7 @@ __device__ __forceinline__ void apply_new(const DPtrs& d, const KParams& p, int 
 // The listed cells first (their chains are the longest), then the commit.
 template <int Q>
 __global__ void __launch_bounds__(kBlock) k_resolve(DPtrs d, KParams p, int parity) {
+  stage_begin();
   const LaneDir l = lane_dir<Q>();
   const int nconv = *conv_count(d);
   for (int j = spread_warp(); j < nconv; j += spread_warps()) resolve_listed<Q>(d, p, parity, l, j);
@@ -408,6 +409,7 @@ __global__ void __launch_bounds__(kBlock) k_resolve(DPtrs d, KParams p, int pari
 
 template <int Q, class S>
 __global__ void __launch_bounds__(kBlock) k_count(DPtrs d, KParams p, int parity) {
+  stage_begin();
   const LaneDir l = lane_dir<Q>();
   const int nconv = *conv_count(d);
   for (int j = spread_warp(); j < nconv; j += spread_warps()) count_listed<Q, S>(d, p, parity, l, j);
@@ -432,12 +434,15 @@ __device__ __forceinline__ void apply_old_items(const DPtrs& d, const KParams& p
   for (int j = first * 32 + l.i; j < nconv; j += stride * 32) apply_converted<S>(d, conv_list(d, parity)[j]);
 }
 
-// The kinds of cells are disjoint and read only what earlier kernels wrote:
-// in one launch, or as two side by side in the step's graph (kNew, kOld:
-// which parts a launch does).  In one launch the new cells (the longest
-// chains) are dealt from the first warp, the others from the last.
+// The kinds of cells are disjoint and read only what earlier kernels wrote
+// (kNew, kOld: which parts a launch does).  In one launch the new cells (the
+// longest chains) are dealt from the first warp, the others from the last.  As
+// two kernels side by side in the graph, the fork and the join cost more than
+// the overlap gave once the stage ran on lists (192^3 drop, a step with the
+// bubbles' fork gone as well: 91.9 us forked, 89.2 in one launch).
 template <int Q, class S, bool kNew, bool kOld>
 __global__ void __launch_bounds__(kBlock) k_apply(DPtrs d, KParams p, int parity) {
+  stage_begin();
   const LaneDir l = lane_dir<Q>();
   const int w = spread_warp(), nw = spread_warps();
   if constexpr (kNew) apply_new_items<Q, S>(d, p, parity, l, w, nw);
@@ -461,6 +466,7 @@ __device__ __forceinline__ void deal_domains(int n, F f) {
 
 template <int Q>
 __global__ void __launch_bounds__(kBlock) kb_resolve(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   const LaneDir l = lane_dir<Q>();
   deal_domains(pl.n, [&](int k, int first, int stride) {
     const DomRec& r = recs[k];
@@ -478,6 +484,7 @@ __global__ void __launch_bounds__(kBlock) kb_resolve(const DomRec* __restrict__ 
 
 template <int Q, class S>
 __global__ void __launch_bounds__(kBlock) kb_count(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   const LaneDir l = lane_dir<Q>();
   deal_domains(pl.n, [&](int k, int first, int stride) {
     const DomRec& r = recs[k];
@@ -489,6 +496,7 @@ __global__ void __launch_bounds__(kBlock) kb_count(const DomRec* __restrict__ re
 // The apply stage of a batch (kNew, kOld as in k_apply).
 template <int Q, class S, bool kNew, bool kOld>
 __global__ void __launch_bounds__(kBlock) kb_apply(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   const LaneDir l = lane_dir<Q>();
   deal_domains(pl.n, [&](int k, int first, int stride) {
     const DomRec& r = recs[k];

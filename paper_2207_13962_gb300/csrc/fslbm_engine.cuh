@@ -79,6 +79,17 @@ struct Engine {
   static void step(const DPtrs& d, const KParams& p, int parity, int band_grid, int bulk_grid,
                    cudaStream_t st, StageEvents* ev, const Fork* fk) {
     const int coll = iface_coll(p);
+    const bool bub = p.bubble_model && d.nb > 0;
+    const bool chained = !ev;  // with an event between two kernels there is nothing to chain
+    // the next list, and the bubble pressures in a block of the same launch (a
+    // launch of its own while stages are timed)
+    auto list_and_bubbles = [&]() {
+      const int beside = bub && !ev;
+      launch_stage(chained, k_compact_band, compact_grid(p, band_grid) + beside, kBlock, 0, st, d, p, parity, beside);
+      if (ev) ev->mark(7, st);
+      if (bub && ev) k_compact_band<<<1, kBlock, 0, st>>>(d, p, parity, 1);
+      if (ev) ev->mark(8, st);
+    };
     if constexpr (kFusedGeo) {
       // geometry and bulk in one persistent launch, then the band chain
       constexpr size_t sm = geometry_smem<typename S::Real>();
@@ -89,41 +100,22 @@ struct Engine {
       with_coll(coll, [&](auto C) { k_bulk_geo<Q, S, decltype(C)::value><<<bulk_grid, kBulkBlock, sm, st>>>(d, p, parity); });
       if (ev) ev->mark(2, st);
       with_coll(coll, [&](auto C) {
-        k_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(d, p, parity);
+        launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity);
       });
       if (ev) ev->mark(3, st);
-      k_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+      launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity);
       if (ev) ev->mark(4, st);
-      k_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+      launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity);
       if (ev) ev->mark(5, st);
-      // the two independent parts of the apply stage, side by side in the
-      // graph (one after the other while stages are timed)
-      const bool side = fk && !ev;
-      if (side) {
-        cudaEventRecord(fk->fork, st);
-        cudaStreamWaitEvent(fk->side, fk->fork, 0);
+      if (ev) {  // its two parts one after the other while stages are timed
+        k_apply<Q, S, true, false><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+        k_apply<Q, S, false, true><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+      } else {
+        launch_stage(chained, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity);
       }
-      k_apply<Q, S, true, false><<<band_grid * 2, kBlock, 0, side ? fk->side : st>>>(d, p, parity);
-      if (side) cudaEventRecord(fk->join, fk->side);
-      k_apply<Q, S, false, true><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
-      if (side) cudaStreamWaitEvent(st, fk->join, 0);
       if (ev) ev->mark(6, st);
-      k_finalize<<<band_grid, kBlock, 0, st>>>(d, p, parity);
-      // the bubble pressures (from finalize's sums) and the list rebuild (from
-      // its flags) are independent: side by side in the graph as well
-      const bool bub = p.bubble_model && d.nb > 0;
-      const bool bub_side = side && bub;
-      if (bub_side) {
-        cudaEventRecord(fk->fork, st);
-        cudaStreamWaitEvent(fk->side, fk->fork, 0);
-        k_bubble<<<1, 256, 0, fk->side>>>(d, p);
-        cudaEventRecord(fk->join, fk->side);
-      }
-      k_compact_band<<<compact_grid(p, band_grid), kBlock, 0, st>>>(d, p, parity);
-      if (ev) ev->mark(7, st);
-      if (bub && !bub_side) k_bubble<<<1, 256, 0, st>>>(d, p);
-      if (bub_side) cudaStreamWaitEvent(st, fk->join, 0);
-      if (ev) ev->mark(8, st);
+      launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity);
+      list_and_bubbles();
       return;
     }
     auto bulk = [&](cudaStream_t s2) {
@@ -151,21 +143,18 @@ struct Engine {
     if (!forked) bulk(st);
     if (ev) ev->mark(2, st);
     with_coll(coll, [&](auto C) {
-      k_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(d, p, parity);
+      launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity);
     });
     if (ev) ev->mark(3, st);
-    k_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+    launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity);
     if (ev) ev->mark(4, st);
-    k_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+    launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity);
     if (ev) ev->mark(5, st);
     if (forked) cudaStreamWaitEvent(st, fk->join, 0);
-    k_apply<Q, S, true, true><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+    launch_stage(chained && !forked, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity);
     if (ev) ev->mark(6, st);
-    k_finalize<<<band_grid, kBlock, 0, st>>>(d, p, parity);
-    k_compact_band<<<compact_grid(p, band_grid), kBlock, 0, st>>>(d, p, parity);
-    if (ev) ev->mark(7, st);
-    if (p.bubble_model && d.nb > 0) k_bubble<<<1, 256, 0, st>>>(d, p);
-    if (ev) ev->mark(8, st);
+    launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity);
+    list_and_bubbles();
   }
 
   // One step of all domains of a block table.  Same stages and stream fork
@@ -176,19 +165,19 @@ struct Engine {
   static void batch_step(DomRec* recs, const BatchPlan& pl, int band_grid, int bulk_grid,
                          int collision, cudaStream_t st, const Fork* fk) {
     kb_plan_front<<<1, 1024, 0, st>>>(recs, pl);
+    constexpr size_t sm = geometry_smem<typename S::Real>();
     if constexpr (kFusedGeo) {
-      constexpr size_t sm = geometry_smem<typename S::Real>();
       with_coll(collision, [&](auto C) {
-        kb_bulk_geo<Q, S, decltype(C)::value><<<bulk_grid, kBulkBlock, sm, st>>>(recs, pl);
+        launch_stage(true, kb_bulk_geo<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, sm, st, recs, pl);
       });
       with_coll(collision, [&](auto C) {
-        kb_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(recs, pl);
+        launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl);
       });
-      kb_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
-      kb_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
-      kb_apply<Q, S, true, true><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
-      kb_finalize<<<band_grid, kBlock, 0, st>>>(recs, pl);
-      kb_bubble_end<<<pl.n, 256, 0, st>>>(recs);
+      launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl);
+      launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl);
+      launch_stage(true, kb_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, recs, pl);
+      launch_stage(true, kb_finalize, band_grid, kBlock, 0, st, recs, pl);
+      launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs);
       (void)fk;
       return;
     }
@@ -198,12 +187,12 @@ struct Engine {
       kb_bulk<Q, S, decltype(C)::value><<<bulk_grid, kBulkBlock, 0, fk->side>>>(recs, pl);
     });
     cudaEventRecord(fk->join, fk->side);
-    kb_geometry<Q, S><<<band_grid * kGeoGridMult, kGeoBlock, geometry_smem<typename S::Real>(), st>>>(recs, pl);
+    kb_geometry<Q, S><<<band_grid * kGeoGridMult, kGeoBlock, sm, st>>>(recs, pl);
     with_coll(collision, [&](auto C) {
-      kb_interface<Q, S, decltype(C)::value><<<band_grid * 2, 128, 0, st>>>(recs, pl);
+      launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl);
     });
-    kb_resolve<Q><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
-    kb_count<Q, S><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
+    launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl);
+    launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl);
     cudaStreamWaitEvent(st, fk->join, 0);
     // the new cells' FP64 chains beside the receivers'
     cudaEventRecord(fk->fork, st);
@@ -213,7 +202,7 @@ struct Engine {
     kb_apply<Q, S, false, true><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
     cudaStreamWaitEvent(st, fk->join, 0);
     kb_finalize<<<band_grid, kBlock, 0, st>>>(recs, pl);
-    kb_bubble_end<<<pl.n, 256, 0, st>>>(recs);
+    launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs);
   }
 
   static void observables(const DPtrs& d, const KParams& p, int parity, double* out,
@@ -276,9 +265,10 @@ struct Engine {
       o.bulk_fn[7] = (const void*)&k_bulk<Q, S, 7>;
     }
     o.bulk_blocks_per_sm = bulk_blocks_per_sm();
-    // bulk and geometry (one launch when fused), interface, resolve,
-    // count, apply (two launches when fused), finalize, list rebuild
-    o.step_launches = 8;
+    // bulk and geometry (one launch when fused), interface, resolve, count,
+    // apply, finalize, list rebuild with the bubbles; while stages are timed
+    // the apply stage is two launches when fused and the bubbles are their own
+    o.step_launches = kFusedGeo ? 7 : 8;
     o.bulk_smem = kTmaBulk ? tma_smem<Q, typename S::T>() : kFusedGeo ? geometry_smem<typename S::Real>() : 0;
     o.batch_step = &batch_step;
     // plan, geometry and bulk sweep (one launch when fused), interface update,

@@ -12,8 +12,8 @@
 //   k_count      list   excess-mass receivers, deferral, shares
 //   k_apply      lists  excess gather, new interface cells' PDFs
 //   k_finalize   band+new  final flags, tile and segment marks, bubble sums
-//   k_compact_band grid the next interface list
-//   k_bubble     1 block   bubble volume pressure
+//   k_compact_band grid the next interface list; in one more block the bubble
+//                       volume pressures
 // The interface work runs only on the compacted list of interface cells
 // ("band") and on the cells that conversion turns into interface cells.
 // Conversion and excess redistribution are gather-only: each cell computes
@@ -798,6 +798,7 @@ __device__ __forceinline__ void reset_step_counts(const DPtrs& d, int parity) {
 
 template <int Q, class S>
 __global__ void __launch_bounds__(kGeoBlock, kGeoMinBlocks) k_geometry(DPtrs d, KParams p, int parity) {
+  stage_begin();
   extern __shared__ __align__(16) unsigned char g_smem[];
   if (blockIdx.x == 0 && threadIdx.x == 0) reset_step_counts(d, parity);
   const int ntiles = d.counts[3 + parity];
@@ -834,6 +835,7 @@ __device__ __forceinline__ void hand_out_tiles(int n, int* counter, int* s_tile,
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     k_bulk_geo(DPtrs d, KParams p, int parity) {
+  stage_begin();
   extern __shared__ __align__(16) unsigned char g_smem[];
   __shared__ int s_tile;
   if (blockIdx.x == 0 && threadIdx.x == 0) reset_step_counts(d, parity);
@@ -1143,6 +1145,7 @@ __device__ __forceinline__ int band_start(int n) {
 
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) k_interface(const __grid_constant__ DPtrs d, const __grid_constant__ KParams p, int parity) {
+  stage_begin();
   const int n = d.counts[parity];
   if (lane_band<Q, S>(n)) {
     interface_by_lanes<Q, S, COLL>(d, p, parity, n);
@@ -1289,6 +1292,7 @@ __device__ __forceinline__ void finalize_lane(const DPtrs& d, const KParams& p, 
 }
 
 static __global__ void __launch_bounds__(kBlock) k_finalize(DPtrs d, KParams p, int parity) {
+  stage_begin();
   const int nband = d.counts[parity], nnew = d.counts[2];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     d.counts[6] = 0;  // the next step's bulk hand-out
@@ -1302,19 +1306,6 @@ static __global__ void __launch_bounds__(kBlock) k_finalize(DPtrs d, KParams p, 
   for (int base = wid * 32; base < nnew; base += warps * 32)
     finalize_lane(d, p, parity, base + lane < nnew ? d.newlist[base + lane] : -1, false);
 }
-
-// p^V_b = p^V_b(0) V_b(0) / V_b (Eq. nm-fslbm-pressure-volume).
-__device__ __forceinline__ void bubble_update(const DPtrs& d, const KParams& p) {
-  for (int b = threadIdx.x; b < d.nb; b += blockDim.x) {
-    const long long acc = d.gas_cnt[b] * 4294967296LL + d.iface_fix[b];
-    const double V = __ll2double_rn(acc) / 4294967296.0;
-    d.pV[b] = (V > 0.0) ? (p.pv0 * d.V0[b]) / V : p.pv0;
-    d.Vcur[b] = V;
-    d.iface_fix[b] = 0;
-  }
-}
-
-static __global__ void k_bubble(DPtrs d, KParams p) { bubble_update(d, p); }
 
 // ------------------------------------------------------------ observables
 // Per-block partials: [0] mass, [1] max|u|^2, [2] liquid volume, [3] nan,
@@ -1535,6 +1526,7 @@ __global__ void k_to_caller(const T* __restrict__ st, T* __restrict__ ext, KPara
 // Plan of the first phase (before geometry): resets the counters this step
 // fills and lays out tiles, bulk warp units and band cells.
 static __global__ void kb_plan_front(DomRec* recs, BatchPlan pl) {
+  stage_begin();
   constexpr int kGroups = 32 / kSegCells;
   if (threadIdx.x == 0) {
     pl.ctr[0] = 0;  // the bulk sweep's hand-out counter
@@ -1549,6 +1541,7 @@ static __global__ void kb_plan_front(DomRec* recs, BatchPlan pl) {
 
 template <int Q, class S>
 __global__ void __launch_bounds__(kGeoBlock, kGeoMinBlocks) kb_geometry(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   extern __shared__ __align__(16) unsigned char g_smem[];
   const int total = pl.tiles[pl.n];
   for (int t = blockIdx.x; t < total; t += gridDim.x) {
@@ -1573,6 +1566,7 @@ __device__ __forceinline__ void batch_bulk_sweep(const DomRec* __restrict__ recs
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     kb_bulk(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   batch_bulk_sweep<Q, S, COLL>(recs, pl);
 }
 
@@ -1582,6 +1576,7 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
     kb_bulk_geo(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   extern __shared__ __align__(16) unsigned char g_smem[];
   __shared__ int s_tile;
   hand_out_tiles(pl.tiles[pl.n], &pl.ctr[1], &s_tile, [&](int t) {
@@ -1594,6 +1589,7 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
 
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) kb_interface(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   const int total = pl.band[pl.n];  // with each domain's cells rounded up to whole warps
   if (lane_band<Q, S>(total)) {
     interface_by_lanes<Q, S, COLL>(recs, pl.band, pl.n, total);
@@ -1611,6 +1607,7 @@ __global__ void __launch_bounds__(128, (iface_min_blocks<S, COLL>())) kb_interfa
 }
 
 static __global__ void __launch_bounds__(kBlock) kb_finalize(const DomRec* __restrict__ recs, BatchPlan pl) {
+  stage_begin();
   const int total = pl.band[pl.n];
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
@@ -1632,6 +1629,7 @@ static __global__ void __launch_bounds__(kBlock) kb_finalize(const DomRec* __res
 // Bubble pressures of every domain (one block each), then the step is done
 // and the domain's buffers swap.
 static __global__ void kb_bubble_end(DomRec* recs) {
+  stage_begin();
   DomRec& r = recs[blockIdx.x];
   if (r.p.bubble_model && r.d.nb > 0) bubble_update(r.d, r.p);
   __syncthreads();
