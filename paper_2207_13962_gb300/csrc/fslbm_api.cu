@@ -798,38 +798,28 @@ fslbm_status fslbm_read_fields(fslbm_ctx* c, double* pdf, double* fill, uint8_t*
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     dfree(c, tmp);
   }
-  if (is_identity_layout(c->kp)) {
-    if (e == cudaSuccess && fill)
-      e = cudaMemcpyAsync(fill, c->d.phi, N * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && mass)
-      e = cudaMemcpyAsync(mass, c->d.mass, N * sizeof(double), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && flags) e = cudaMemcpyAsync(flags, c->d.flags, N, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  } else if (e == cudaSuccess && (fill || mass || flags)) {
-    // the fields in the caller's cell order, through one staging array
-    double* tmp = nullptr;
-    e = dalloc(c, &tmp, N * sizeof(double));
+  // Fill levels, masses and types in the caller's cell order, staged in arrays
+  // that are idle between steps, then copied with one wait at the end.  The
+  // types lose their static bits on the device.  Staging in an allocated array
+  // and masking the bytes on the host: 160x160x1024 tube 4.4 ms (0.45 GB).
+  if (e == cudaSuccess && (fill || mass || flags)) {
     const int grid = (c->kp.N + kBlock - 1) / kBlock;
-    auto out = [&](const double* src, double* host) {
-      if (e != cudaSuccess || !host) return;
-      k_to_caller<double><<<grid, kBlock, 0, st>>>(src, tmp, c->kp);
-      e = cudaGetLastError();
-      if (e == cudaSuccess) e = cudaMemcpyAsync(host, tmp, N * sizeof(double), cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    };
-    out(c->d.phi, fill);
-    out(c->d.mass, mass);
-    if (e == cudaSuccess && flags) {
-      k_to_caller<uint8_t><<<grid, kBlock, 0, st>>>(c->d.flags, (uint8_t*)tmp, c->kp);
-      e = cudaGetLastError();
-      if (e == cudaSuccess) e = cudaMemcpyAsync(flags, tmp, N, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const double *phi_out = c->d.phi, *mass_out = c->d.mass;
+    uint8_t* types_out = (uint8_t*)c->d.nhat;
+    if (!is_identity_layout(c->kp)) {
+      if (fill) k_to_caller<double><<<grid, kBlock, 0, st>>>(c->d.phi, c->d.phi_next, c->kp);
+      if (mass) k_to_caller<double><<<grid, kBlock, 0, st>>>(c->d.mass, c->d.m_next, c->kp);
+      phi_out = c->d.phi_next;
+      mass_out = c->d.m_next;
     }
-    dfree(c, tmp);
+    if (flags) k_types_to_caller<<<grid, kBlock, 0, st>>>(c->d.flags, types_out, c->kp);
+    e = cudaGetLastError();
+    if (e == cudaSuccess && fill) e = cudaMemcpyAsync(fill, phi_out, N * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && mass) e = cudaMemcpyAsync(mass, mass_out, N * sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && flags) e = cudaMemcpyAsync(flags, types_out, N, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }
   if (e != cudaSuccess) return cuda_fail(c, e, "fslbm_read_fields");
-  if (flags)
-    for (size_t i = 0; i < N; ++i) flags[i] &= F_TYPE;
   return FSLBM_OK;
 }
 

@@ -1514,6 +1514,12 @@ __global__ void k_to_caller(const T* __restrict__ st, T* __restrict__ ext, KPara
   ext[e] = st[storage_of_ext(p, e)];
 }
 
+// Cell types of the flags in the caller's cell order.
+static __global__ void k_types_to_caller(const uint8_t* __restrict__ flags, uint8_t* __restrict__ ext, KParams p) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < p.N) ext[e] = flags[storage_of_ext(p, e)] & F_TYPE;
+}
+
 // ---------------------------------------------------------------- batches
 // Many domains of different sizes advance in one launch per phase.  The
 // block table is an array of DomRec; the plan kernels turn each domain's
