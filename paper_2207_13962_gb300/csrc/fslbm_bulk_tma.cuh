@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kBulkBlock, kBulkMinBlocks32) k_bulk_tma(DPtrs
         }
         bulk_finish<Q, S, COLL>(d, p, parity, c, fl, f);
       } else {
-        bulk_cell<Q, S, COLL>(d, p, parity, c, fl, true);
+        bulk_cell<Q, S, COLL>(d, p, parity, c, fl, kWrap);
       }
     } else if (FSLBM_BULK_FILL) {
       constexpr int kFill = 32 / (int)sizeof(T);
