@@ -52,6 +52,13 @@ int max_bulk_blocks(const fslbm_batch* b) {
   return (b->collision & 2) ? 3 : kBulkMinBlocks32;  // the Smagorinsky sweep is compiled for 3
 }
 
+// Resident blocks per SM the batch starts with: as many as its sweep is
+// compiled for (bulk_min_blocks).
+int default_bulk_blocks(const fslbm_batch* b) {
+  const int most = max_bulk_blocks(b);
+  return b->ops.rest_size && b->m[0]->q == 27 && most > 3 ? 3 : most;
+}
+
 cudaError_t capture(fslbm_batch* b) {
   if (b->graph) {
     cudaGraphExecDestroy(b->graph);
@@ -140,7 +147,7 @@ fslbm_status fslbm_batch_create(fslbm_ctx* const* members, int n, void* stream, 
   int dev = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) b->sms = 152;
-  b->tune.bulk_blocks_per_sm = max_bulk_blocks(b);
+  b->tune.bulk_blocks_per_sm = default_bulk_blocks(b);
   b->tune.band_blocks_per_sm = 2;
   b->tune.ms_per_step = 0.0;
   cudaError_t e = cudaMalloc(&b->d_recs, (size_t)n * sizeof(DomRec));

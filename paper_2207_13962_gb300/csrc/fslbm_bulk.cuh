@@ -213,10 +213,13 @@ __device__ __forceinline__ void hand_out_units(int n, int* counter, F unit) {
 
 // Resident blocks per SM a bulk sweep is compiled for: the FP32 engines
 // kBulkMinBlocks32 (64 registers), 3 with the Smagorinsky model (its
-// momentum flux needs more), the FP64 engine 2.
-template <class S, int COLL>
+// momentum flux needs more) and in the mass-conserving formats with 27
+// directions (8 cylinders in FP16SMC, a step: 128 us, 131 with four blocks;
+// with 19 directions three lose, 96x96x384 tube 121 against 115), the FP64
+// engine 2.
+template <int Q, class S, int COLL>
 constexpr int bulk_min_blocks() {
-  return sizeof(typename S::Real) == 4 ? (coll_les(COLL) ? 3 : kBulkMinBlocks32) : 2;
+  return sizeof(typename S::Real) == 4 ? (coll_les(COLL) || (S::kExactRest && Q == 27) ? 3 : kBulkMinBlocks32) : 2;
 }
 
 // The sweep over the liquid segments by the warps of a persistent grid.
@@ -229,7 +232,7 @@ __device__ __forceinline__ void bulk_sweep(const DPtrs& d, const KParams& p, int
 }
 
 template <int Q, class S, int COLL>
-__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
+__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<Q, S, COLL>()))
     k_bulk(DPtrs d, KParams p, int parity) {
   stage_begin();
   bulk_sweep<Q, S, COLL>(d, p, parity);

@@ -833,7 +833,7 @@ __device__ __forceinline__ void hand_out_tiles(int n, int* counter, int* s_tile,
 // its blocks to keep HBM busy, so blocks held by tiles slow it by about what
 // running the tiles beside it saves.
 template <int Q, class S, int COLL>
-__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
+__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<Q, S, COLL>()))
     k_bulk_geo(DPtrs d, KParams p, int parity) {
   stage_begin();
   extern __shared__ __align__(16) unsigned char g_smem[];
@@ -1577,7 +1577,7 @@ __device__ __forceinline__ void batch_bulk_sweep(const DomRec* __restrict__ recs
 }
 
 template <int Q, class S, int COLL>
-__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
+__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<Q, S, COLL>()))
     kb_bulk(const DomRec* __restrict__ recs, BatchPlan pl) {
   stage_begin();
   batch_bulk_sweep<Q, S, COLL>(recs, pl);
@@ -1587,7 +1587,7 @@ __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
 // as k_bulk_geo: the blocks first take tiles from the plan's tile counter,
 // then bulk units.
 template <int Q, class S, int COLL>
-__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<S, COLL>()))
+__global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<Q, S, COLL>()))
     kb_bulk_geo(const DomRec* __restrict__ recs, BatchPlan pl) {
   stage_begin();
   extern __shared__ __align__(16) unsigned char g_smem[];
