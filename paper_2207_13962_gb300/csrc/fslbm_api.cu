@@ -105,19 +105,13 @@ void destroy_graphs(fslbm_ctx* c) {
 
 cudaError_t build_graphs(fslbm_ctx* c) {
   destroy_graphs(c);
-  for (int par = 0; par < 2; ++par) {
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return e;
-    c->ops.step(c->d, c->kp, par, c->band_grid, c->bulk_grid, c->cap_stream, nullptr, &c->fork);
-    e = cudaStreamEndCapture(c->cap_stream, &g);
-    if (e != cudaSuccess) return e;
-    e = prioritise_nodes(g, c->ops.bulk_fn[coll_of(c->kp) | slip_bit(c->kp)], nullptr);
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph[par], g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  for (int par = 0; par < 2 && e == cudaSuccess; ++par)
+    e = capture_graph(c->cap_stream, &c->graph[par], c->ops.bulk_fn[coll_of(c->kp) | slip_bit(c->kp)], [&]() {
+      return c->ops.step(c->d, c->kp, par, c->band_grid, c->bulk_grid, c->cap_stream, nullptr, &c->fork);
+    });
+  if (e != cudaSuccess) destroy_graphs(c);
+  return e;
 }
 
 int launches_per_step(const fslbm_ctx* c) {
@@ -714,8 +708,7 @@ fslbm_status fslbm_step(fslbm_ctx* c, int n) {
   for (int s = 0; s < n; ++s) {
     cudaError_t e;
     if (c->timing) {
-      c->ops.step(c->d, c->kp, c->parity, c->band_grid, c->bulk_grid, c->stream, &c->ev, nullptr);
-      e = cudaGetLastError();
+      e = c->ops.step(c->d, c->kp, c->parity, c->band_grid, c->bulk_grid, c->stream, &c->ev, nullptr);
       if (e == cudaSuccess) e = cudaEventSynchronize(c->ev.ev[StageEvents::kMarks - 1]);
       if (e == cudaSuccess) {
         for (int k = 0; k < StageEvents::kStages; ++k) {

@@ -64,20 +64,15 @@ cudaError_t capture(fslbm_batch* b) {
     cudaGraphExecDestroy(b->graph);
     b->graph = nullptr;
   }
-  cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
-  if (e != cudaSuccess) return e;
-  b->ops.batch_step(b->d_recs, b->plan, b->sms * b->tune.band_blocks_per_sm,
-                    b->sms * b->tune.bulk_blocks_per_sm, b->collision, b->cap, &b->fork);
-  // every member's next interface list in cell order
-  launch_stage(true, kb_compact_band, b->nchunks < 8 * b->sms ? b->nchunks : 8 * b->sms, kBlock, 0, b->cap,
-               b->d_recs, b->d_chunk, (int)b->m.size());
-  e = cudaStreamEndCapture(b->cap, &g);
-  if (e != cudaSuccess) return e;
-  e = prioritise_nodes(g, b->ops.batch_bulk_fn[b->collision], nullptr);
-  if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph, g, 0);
-  cudaGraphDestroy(g);
-  return e;
+  return capture_graph(b->cap, &b->graph, b->ops.batch_bulk_fn[b->collision], [&]() {
+    FirstError keep;
+    keep(b->ops.batch_step(b->d_recs, b->plan, b->sms * b->tune.band_blocks_per_sm,
+                           b->sms * b->tune.bulk_blocks_per_sm, b->collision, b->cap, &b->fork));
+    // every member's next interface list in cell order
+    keep(launch_stage(true, kb_compact_band, b->nchunks < 8 * b->sms ? b->nchunks : 8 * b->sms, kBlock, 0, b->cap,
+                      b->d_recs, b->d_chunk, (int)b->m.size()));
+    return keep.e;
+  });
 }
 
 // Upload the block table (each member's pointers, parameters and current

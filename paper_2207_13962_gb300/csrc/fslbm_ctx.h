@@ -53,4 +53,23 @@ namespace fslbm {
 fslbm_status fail(fslbm_ctx* c, fslbm_status s, const std::string& msg);
 fslbm_status cuda_fail(fslbm_ctx* c, cudaError_t e, const char* where);
 cudaError_t prioritise_nodes(cudaGraph_t g, const void* skip0, const void* skip1);
+
+// Captures the launches that `enqueue` makes on st into an executable graph.
+// enqueue returns the first error of its launches; with one, there is no graph
+// (the capture itself can succeed without the rejected launch).  The node of
+// kernel bulk_fn keeps the default priority.
+template <class F>
+cudaError_t capture_graph(cudaStream_t st, cudaGraphExec_t* out, const void* bulk_fn, F enqueue) {
+  cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
+  e = enqueue();
+  cudaGraph_t g = nullptr;
+  const cudaError_t ended = cudaStreamEndCapture(st, &g);
+  if (e == cudaSuccess) e = ended;
+  if (e == cudaSuccess) e = prioritise_nodes(g, bulk_fn, nullptr);
+  if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+  if (g) cudaGraphDestroy(g);
+  if (e != cudaSuccess) cudaGetLastError();  // reported by the return value
+  return e;
+}
 }  // namespace fslbm

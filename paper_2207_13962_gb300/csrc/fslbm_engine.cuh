@@ -72,12 +72,14 @@ struct Engine {
   }
 
   // One step reading pdf[parity], band[parity]; writing the other buffers.
+  // Returns the first error of its launches.
   // With a Fork (and no stage events) the bulk sweep runs on the side stream
   // while geometry, interface update and the first conversion passes run on
   // the main stream; the streams join before k_apply, the first kernel that
   // reads post-collision PDFs of liquid cells.
-  static void step(const DPtrs& d, const KParams& p, int parity, int band_grid, int bulk_grid,
-                   cudaStream_t st, StageEvents* ev, const Fork* fk) {
+  static cudaError_t step(const DPtrs& d, const KParams& p, int parity, int band_grid, int bulk_grid,
+                          cudaStream_t st, StageEvents* ev, const Fork* fk) {
+    FirstError keep;
     const int coll = iface_coll(p);
     const bool bub = p.bubble_model && d.nb > 0;
     const bool chained = !ev;  // with an event between two kernels there is nothing to chain
@@ -85,9 +87,10 @@ struct Engine {
     // launch of its own while stages are timed)
     auto list_and_bubbles = [&]() {
       const int beside = bub && !ev;
-      launch_stage(chained, k_compact_band, compact_grid(p, band_grid) + beside, kBlock, 0, st, d, p, parity, beside);
+      keep(launch_stage(chained, k_compact_band, compact_grid(p, band_grid) + beside, kBlock, 0, st, d, p, parity,
+                        beside));
       if (ev) ev->mark(7, st);
-      if (bub && ev) k_compact_band<<<1, kBlock, 0, st>>>(d, p, parity, 1);
+      if (bub && ev) keep(launch_stage(false, k_compact_band, 1, kBlock, 0, st, d, p, parity, 1));
       if (ev) ev->mark(8, st);
     };
     if constexpr (kFusedGeo) {
@@ -97,64 +100,68 @@ struct Engine {
         ev->mark(0, st);
         ev->mark(1, st);
       }
-      with_coll(coll, [&](auto C) { k_bulk_geo<Q, S, decltype(C)::value><<<bulk_grid, kBulkBlock, sm, st>>>(d, p, parity); });
+      with_coll(coll, [&](auto C) {
+        keep(launch_stage(false, k_bulk_geo<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, sm, st, d, p, parity));
+      });
       if (ev) ev->mark(2, st);
       with_coll(coll, [&](auto C) {
-        launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity);
+        keep(launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity));
       });
       if (ev) ev->mark(3, st);
-      launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity);
+      keep(launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity));
       if (ev) ev->mark(4, st);
-      launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity);
+      keep(launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity));
       if (ev) ev->mark(5, st);
       if (ev) {  // its two parts one after the other while stages are timed
-        k_apply<Q, S, true, false><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
-        k_apply<Q, S, false, true><<<band_grid * 2, kBlock, 0, st>>>(d, p, parity);
+        keep(launch_stage(false, k_apply<Q, S, true, false>, band_grid * 2, kBlock, 0, st, d, p, parity));
+        keep(launch_stage(false, k_apply<Q, S, false, true>, band_grid * 2, kBlock, 0, st, d, p, parity));
       } else {
-        launch_stage(chained, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity);
+        keep(launch_stage(chained, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity));
       }
       if (ev) ev->mark(6, st);
-      launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity);
+      keep(launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity));
       list_and_bubbles();
-      return;
+      return keep.e;
     }
     auto bulk = [&](cudaStream_t s2) {
       with_coll(coll, [&](auto C) {
         constexpr int CO = decltype(C)::value;
         if constexpr (kTmaBulk && !coll_les(CO)) {
           constexpr size_t sm = tma_smem<Q, typename S::T>();
-          k_bulk_tma<Q, S, CO><<<bulk_grid, kBulkBlock, sm, s2>>>(d, p, parity);
+          keep(launch_stage(false, k_bulk_tma<Q, S, CO>, bulk_grid, kBulkBlock, sm, s2, d, p, parity));
         } else {
-          k_bulk<Q, S, CO><<<bulk_grid, kBulkBlock, 0, s2>>>(d, p, parity);
+          keep(launch_stage(false, k_bulk<Q, S, CO>, bulk_grid, kBulkBlock, 0, s2, d, p, parity));
         }
       });
     };
     const bool forked = fk && !ev;
     auto fork_bulk = [&]() {
-      cudaEventRecord(fk->fork, st);
-      cudaStreamWaitEvent(fk->side, fk->fork, 0);
+      keep(cudaEventRecord(fk->fork, st));
+      keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
       bulk(fk->side);
-      cudaEventRecord(fk->join, fk->side);
+      keep(cudaEventRecord(fk->join, fk->side));
     };
     if (ev) ev->mark(0, st);
     if (forked) fork_bulk();
-    k_geometry<Q, S><<<band_grid * kGeoGridMult, kGeoBlock, geometry_smem<typename S::Real>(), st>>>(d, p, parity);
+    keep(launch_stage(false, k_geometry<Q, S>, band_grid * kGeoGridMult, kGeoBlock,
+                      geometry_smem<typename S::Real>(), st, d, p, parity));
     if (ev) ev->mark(1, st);
     if (!forked) bulk(st);
     if (ev) ev->mark(2, st);
     with_coll(coll, [&](auto C) {
-      launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity);
+      keep(launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity));
     });
     if (ev) ev->mark(3, st);
-    launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity);
+    keep(launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity));
     if (ev) ev->mark(4, st);
-    launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity);
+    keep(launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity));
     if (ev) ev->mark(5, st);
-    if (forked) cudaStreamWaitEvent(st, fk->join, 0);
-    launch_stage(chained && !forked, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity);
+    if (forked) keep(cudaStreamWaitEvent(st, fk->join, 0));
+    keep(launch_stage(chained && !forked, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity));
     if (ev) ev->mark(6, st);
-    launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity);
+    keep(launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity));
     list_and_bubbles();
+    return keep.e;
   }
 
   // One step of all domains of a block table.  Same stages and stream fork
@@ -162,47 +169,49 @@ struct Engine {
   // the last kernel swaps every domain's buffers.  collision: the variant
   // shared by the members (coll_of), with bit 2 set when one of them has
   // free-slip faces.
-  static void batch_step(DomRec* recs, const BatchPlan& pl, int band_grid, int bulk_grid,
-                         int collision, cudaStream_t st, const Fork* fk) {
-    kb_plan_front<<<1, 1024, 0, st>>>(recs, pl);
+  static cudaError_t batch_step(DomRec* recs, const BatchPlan& pl, int band_grid, int bulk_grid,
+                                int collision, cudaStream_t st, const Fork* fk) {
+    FirstError keep;
+    keep(launch_stage(false, kb_plan_front, 1, 1024, 0, st, recs, pl));
     constexpr size_t sm = geometry_smem<typename S::Real>();
     if constexpr (kFusedGeo) {
       with_coll(collision, [&](auto C) {
-        launch_stage(true, kb_bulk_geo<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, sm, st, recs, pl);
+        keep(launch_stage(true, kb_bulk_geo<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, sm, st, recs, pl));
       });
       with_coll(collision, [&](auto C) {
-        launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl);
+        keep(launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl));
       });
-      launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl);
-      launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl);
-      launch_stage(true, kb_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, recs, pl);
-      launch_stage(true, kb_finalize, band_grid, kBlock, 0, st, recs, pl);
-      launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs);
+      keep(launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl));
+      keep(launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl));
+      keep(launch_stage(true, kb_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, recs, pl));
+      keep(launch_stage(true, kb_finalize, band_grid, kBlock, 0, st, recs, pl));
+      keep(launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs));
       (void)fk;
-      return;
+      return keep.e;
     }
-    cudaEventRecord(fk->fork, st);
-    cudaStreamWaitEvent(fk->side, fk->fork, 0);
+    keep(cudaEventRecord(fk->fork, st));
+    keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
     with_coll(collision, [&](auto C) {
-      kb_bulk<Q, S, decltype(C)::value><<<bulk_grid, kBulkBlock, 0, fk->side>>>(recs, pl);
+      keep(launch_stage(false, kb_bulk<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, 0, fk->side, recs, pl));
     });
-    cudaEventRecord(fk->join, fk->side);
-    kb_geometry<Q, S><<<band_grid * kGeoGridMult, kGeoBlock, sm, st>>>(recs, pl);
+    keep(cudaEventRecord(fk->join, fk->side));
+    keep(launch_stage(false, kb_geometry<Q, S>, band_grid * kGeoGridMult, kGeoBlock, sm, st, recs, pl));
     with_coll(collision, [&](auto C) {
-      launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl);
+      keep(launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl));
     });
-    launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl);
-    launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl);
-    cudaStreamWaitEvent(st, fk->join, 0);
+    keep(launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl));
+    keep(launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl));
+    keep(cudaStreamWaitEvent(st, fk->join, 0));
     // the new cells' FP64 chains beside the receivers'
-    cudaEventRecord(fk->fork, st);
-    cudaStreamWaitEvent(fk->side, fk->fork, 0);
-    kb_apply<Q, S, true, false><<<band_grid * 2, kBlock, 0, fk->side>>>(recs, pl);
-    cudaEventRecord(fk->join, fk->side);
-    kb_apply<Q, S, false, true><<<band_grid * 2, kBlock, 0, st>>>(recs, pl);
-    cudaStreamWaitEvent(st, fk->join, 0);
-    kb_finalize<<<band_grid, kBlock, 0, st>>>(recs, pl);
-    launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs);
+    keep(cudaEventRecord(fk->fork, st));
+    keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
+    keep(launch_stage(false, kb_apply<Q, S, true, false>, band_grid * 2, kBlock, 0, fk->side, recs, pl));
+    keep(cudaEventRecord(fk->join, fk->side));
+    keep(launch_stage(false, kb_apply<Q, S, false, true>, band_grid * 2, kBlock, 0, st, recs, pl));
+    keep(cudaStreamWaitEvent(st, fk->join, 0));
+    keep(launch_stage(false, kb_finalize, band_grid, kBlock, 0, st, recs, pl));
+    keep(launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs));
+    return keep.e;
   }
 
   static void observables(const DPtrs& d, const KParams& p, int parity, double* out,

@@ -30,8 +30,12 @@ struct Fork {
 // launch is prepared while that one drains (see stage_begin).  Seven
 // boundaries of a step: 37x21x11 tank 51.9 -> 49.6 us a step, 256x128x64 dam
 // break 60.0 -> 58.6, 32x64x1 FP64 wave 51.9 -> 50.3.
+//
+// A launch that is rejected does not always invalidate the capture it is part
+// of, so a graph can be complete but for one stage: every launch of a step
+// reports its status, and a step with a failed one is not made into a graph.
 template <class... P, class... A>
-inline void launch_stage(bool chained, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
+inline cudaError_t launch_stage(bool chained, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
                          A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
@@ -43,8 +47,16 @@ inline void launch_stage(bool chained, void (*kernel)(P...), int grid, int block
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = chained ? 1u : 0u;
-  cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);
 }
+
+// The first error of a sequence of calls.
+struct FirstError {
+  cudaError_t e = cudaSuccess;
+  void operator()(cudaError_t r) {
+    if (e == cudaSuccess) e = r;
+  }
+};
 
 struct Ops {
   void (*init_cells)(const DPtrs&, const KParams&, const uint8_t* raw, const double* fill,
@@ -54,8 +66,9 @@ struct Ops {
   void (*cc_union)(const uint8_t* raw, const KParams&, int* lab, cudaStream_t);
   void (*cc_assign)(const uint8_t* raw, const KParams&, const int* lab, const int* root_id,
                     int* bid, cudaStream_t);
-  void (*step)(const DPtrs&, const KParams&, int parity, int band_grid, int bulk_grid,
-               cudaStream_t, StageEvents*, const Fork*);
+  // the kernels of one step; the first error of their launches
+  cudaError_t (*step)(const DPtrs&, const KParams&, int parity, int band_grid, int bulk_grid,
+                      cudaStream_t, StageEvents*, const Fork*);
   void (*observables)(const DPtrs&, const KParams&, int parity, double* out, cudaStream_t);
   void (*pdf_out)(const DPtrs&, const KParams&, int parity, double* out, cudaStream_t);
   size_t elem_size;
@@ -68,8 +81,8 @@ struct Ops {
   size_t bulk_smem;        // its dynamic shared memory per block
   int step_launches;       // kernels one step launches from its graph
   // one step of every domain of a block table (see DomRec, BatchPlan)
-  void (*batch_step)(DomRec* recs, const BatchPlan& plan, int band_grid, int bulk_grid,
-                     int collision, cudaStream_t, const Fork*);
+  cudaError_t (*batch_step)(DomRec* recs, const BatchPlan& plan, int band_grid, int bulk_grid,
+                            int collision, cudaStream_t, const Fork*);
   const void* batch_bulk_fn[8];
   int batch_step_launches;  // kernels one batched step launches
 };
