@@ -319,8 +319,13 @@ fslbm_status fslbm_memory_estimate(const fslbm_domain* domain, fslbm_lattice lat
   size_t b = 2 * ((size_t)lattice * Np * elem + Np * rest);  // PDFs, two buffers
   b += 6 * n4 + (N + 31) / 32 * 32;                      // cls, mark, conv, cfin, claim, rcv; flags
   b += N * (4 + 8 + 8 + 4 + 8 + 4 + 4 + 4);              // wallmask phi mass bid share band[2] newlist
-  b += N * (7 * rs + 4 * 8);                             // nhat rhog mom m_next phi_next rho_band
-  b += 3 * ntiles * 4 + 2 * nseg * 4 + 4096;             // tiles, segments, counters, partials
+  b += N * (7 * rs + 3 * 8);                             // nhat rhog mom_u; mom_rho m_next phi_next
+  b += N * (rs == 8 ? 8 : 4);                            // rho_band (FP64), phif (the others)
+  b += 3 * ntiles * 4 + 2 * nseg * 4;                    // tiles, segments
+  // partials of the observables on up to 256 SMs; counters, results and the
+  // arrays of some 64 bubbles
+  b += (size_t)256 * kObsBlocksPerSm * kObsFields * sizeof(double) + 4096;
+  b += (N / kCcChunk + 2) * 2 * sizeof(int);             // bubble numbering at init
   b += 2 * (N * (1 + 8 + 8) + (with_velocity ? 24 * N : 0));  // fslbm_init staging in the
                                                            // caller's and the storage order
   *bytes = b;

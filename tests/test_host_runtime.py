@@ -85,3 +85,27 @@ missed = [k for k in range(8) if not fails(lambda: c.step(1), k)]
 assert not missed, missed
 c.step(1)
 """)
+
+
+@pytest.mark.parametrize("precision", ["FP64", "FP32", "FP16S", "BF16S", "FP32MC", "FP16SMC"])
+def test_memory_estimate_covers_what_a_context_takes(run, precision):
+    """The admission estimate against the bytes that create and init allocate
+    at most, with every array staged twice: never less, and above it by no
+    more than the partials of the SMs the device does not have (the estimate
+    allows for 256 SMs), the bubbles it allows for and the small change."""
+    run(f"""
+for q in (19, 27):
+    for shape in ((1, 1, 1), (3, 2, 1), (40, 9, 5), (64, 33, 17)):
+        n = shape[0] * shape[1] * shape[2]
+        for sms in (152, 256):
+            var("fake_sms").value = sms
+            base = var("fake_bytes", ctypes.c_size_t).value
+            var("fake_peak", ctypes.c_size_t).value = base
+            c = context({precision!r}, shape=shape, q=q, bubble_model=True, vel=np.zeros(3 * n), den=np.ones(n),
+                        axis_order=(2, 1, 0))
+            took = var("fake_peak", ctypes.c_size_t).value - base
+            c.close()
+            est = fslbm.memory_estimate(shape, q, {precision!r}, with_velocity=True)
+            slack = (256 - sms) * 4 * 8 * 8 + 8192
+            assert took <= est <= took + slack, (q, shape, sms, took, est)
+""")
