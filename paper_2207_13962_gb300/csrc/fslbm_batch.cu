@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "fslbm_band_list.cuh"
+#include "fslbm_bulk.cuh"
 #include "fslbm_ctx.h"
 
 using namespace fslbm;
@@ -29,6 +30,7 @@ struct fslbm_batch {
   std::vector<DomRec> h_recs;
   cudaGraphExec_t graph = nullptr;
   int sms = 152;
+  int bulk_fit = 0;                // resident blocks per SM of the bulk sweep (0: unknown)
   fslbm_tuning tune{};
   long long launches = 0;          // kernels launched by batch steps
   std::string err;
@@ -52,11 +54,13 @@ int max_bulk_blocks(const fslbm_batch* b) {
   return (b->collision & 2) ? 3 : kBulkMinBlocks32;  // the Smagorinsky sweep is compiled for 3
 }
 
-// Resident blocks per SM the batch starts with: as many as its sweep is
-// compiled for (bulk_min_blocks).
-int default_bulk_blocks(const fslbm_batch* b) {
-  const int most = max_bulk_blocks(b);
-  return b->ops.rest_size && b->m[0]->q == 27 && most > 3 ? 3 : most;
+// Blocks of the persistent bulk sweep per SM that are launched for a tuning of
+// `blocks`: no more than can be resident at once (what the kernel of this
+// lattice, format and collision is compiled for, as fslbm_create does for one
+// domain).  A block that has to wait for another one to end would still own the
+// first tile and the first units of its number, and they would come last.
+int launched_bulk_blocks(const fslbm_batch* b, int blocks) {
+  return b->bulk_fit > 0 && b->bulk_fit < blocks ? b->bulk_fit : blocks;
 }
 
 cudaError_t capture(fslbm_batch* b) {
@@ -67,7 +71,7 @@ cudaError_t capture(fslbm_batch* b) {
   return capture_graph(b->cap, &b->graph, b->ops.batch_bulk_fn[b->collision], [&]() {
     FirstError keep;
     keep(b->ops.batch_step(b->d_recs, b->plan, b->sms * b->tune.band_blocks_per_sm,
-                           b->sms * b->tune.bulk_blocks_per_sm, b->collision, b->cap, &b->fork));
+                           b->sms * launched_bulk_blocks(b, b->tune.bulk_blocks_per_sm), b->collision, b->cap, &b->fork));
     // every member's next interface list in cell order
     keep(launch_stage(true, kb_compact_band, b->nchunks < 8 * b->sms ? b->nchunks : 8 * b->sms, kBlock, 0, b->cap,
                       b->d_recs, b->d_chunk, (int)b->m.size()));
@@ -142,7 +146,12 @@ fslbm_status fslbm_batch_create(fslbm_ctx* const* members, int n, void* stream, 
   int dev = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) b->sms = 152;
-  b->tune.bulk_blocks_per_sm = default_bulk_blocks(b);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->bulk_fit, b->ops.batch_bulk_fn[b->collision], kBulkBlock,
+                                                    b->ops.bulk_smem) != cudaSuccess) {
+    b->bulk_fit = 0;
+    cudaGetLastError();
+  }
+  b->tune.bulk_blocks_per_sm = launched_bulk_blocks(b, max_bulk_blocks(b));
   b->tune.band_blocks_per_sm = 2;
   b->tune.ms_per_step = 0.0;
   cudaError_t e = cudaMalloc(&b->d_recs, (size_t)n * sizeof(DomRec));
@@ -235,7 +244,8 @@ fslbm_status fslbm_batch_autotune(fslbm_batch* b, int steps, fslbm_tuning* chose
   fslbm_tuning best = b->tune;
   best.ms_per_step = -1.0;
   const int band_opts[4] = {1, 2, 4, 8};
-  for (int bulk = 1; bulk <= max_bulk_blocks(b) && e == cudaSuccess; ++bulk) {
+  const int most = launched_bulk_blocks(b, max_bulk_blocks(b));
+  for (int bulk = 1; bulk <= most && e == cudaSuccess; ++bulk) {
     for (int oi = 0; oi < 4 && e == cudaSuccess; ++oi) {
       b->tune.bulk_blocks_per_sm = bulk;
       b->tune.band_blocks_per_sm = band_opts[oi];

@@ -109,3 +109,35 @@ for q in (19, 27):
             slack = (256 - sms) * 4 * 8 * 8 + 8192
             assert took <= est <= took + slack, (q, shape, sms, took, est)
 """)
+
+
+@pytest.mark.parametrize("precision,most", [("FP64", 2), ("FP32", 4), ("FP16SMC", 4)])
+@pytest.mark.parametrize("fit", [1, 2, 3, 4, 9])
+def test_a_batch_launches_no_more_sweep_blocks_than_fit(run, precision, most, fit):
+    """Every tuning up to the format's limit is accepted; the persistent sweep
+    gets that many blocks per SM, or as many as can be resident at once."""
+    run(f"""
+var("fake_occupancy").value = {fit}
+members = [context({precision!r}, q=27) for _ in range(2)]
+block, grid = (ctypes.c_uint * 4096).in_dll(fake, "fake_block"), (ctypes.c_uint * 4096).in_dll(fake, "fake_grid")
+def sweep(call):
+    first = var("fake_launches").value
+    out = call()
+    k = first + 1  # after the plan kernel
+    assert block[k] == 256
+    return out, grid[k]
+b, g = sweep(lambda: fslbm.Batch(members))
+assert g == 152 * min({most}, {fit}), g
+assert b.tuning()["bulk_blocks_per_sm"] == min({most}, {fit})
+for t in range(1, {most} + 1):
+    _, g = sweep(lambda: b.set_tuning(t, 2))
+    assert g == 152 * min(t, {fit}), (t, g)
+    assert b.tuning()["bulk_blocks_per_sm"] == t
+for t in (0, {most} + 1):
+    try:
+        b.set_tuning(t, 2)
+    except fslbm.FslbmError as e:
+        assert e.status == fslbm.EINVAL
+    else:
+        raise AssertionError(t)
+""")
