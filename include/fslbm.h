@@ -47,7 +47,8 @@ typedef enum {
   FSLBM_ECUDA = 3,      /* a CUDA call failed; see fslbm_last_error()        */
   FSLBM_EUNSTABLE = 4,  /* |u|^2 >= c_s^2, rho <= 0 or a NaN was seen
                            (the instability of Sec. 4.2); fields stay readable */
-  FSLBM_ETIMEOUT = 5,   /* a bounded device wait gave up                     */
+  FSLBM_ETIMEOUT = 5,   /* a bounded device wait gave up (no kernel of this
+                           version waits on the device: never returned)       */
   FSLBM_ESTATE = 6,     /* call out of order (e.g. step before init)         */
   FSLBM_ECAPACITY = 7   /* a list outgrew its capacity (not returned: the
                            interface and new-cell lists hold every cell) */
@@ -200,9 +201,7 @@ fslbm_status fslbm_init(fslbm_ctx* ctx, const double* fill, const uint8_t* flags
  * instability is reported by fslbm_sync / fslbm_observables. */
 fslbm_status fslbm_step(fslbm_ctx* ctx, int n);
 
-/* Wait for the stream; FSLBM_EUNSTABLE if an instability was flagged,
- * FSLBM_ETIMEOUT if a bounded device wait gave up (only the TMA-staged bulk
- * sweep waits on the device; it is not built by default). */
+/* Wait for the stream; FSLBM_EUNSTABLE if an instability was flagged. */
 fslbm_status fslbm_sync(fslbm_ctx* ctx);
 
 /* Whole-domain observables; synchronizes.  Returns FSLBM_EUNSTABLE (with

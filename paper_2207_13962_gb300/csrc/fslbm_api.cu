@@ -240,9 +240,8 @@ fslbm_status fslbm_create(const fslbm_domain* domain, fslbm_lattice lattice,
   if (e == cudaSuccess) e = dalloc(c, &(ptr), (bytes));
   ALLOC(d.pdf[0], pdf_bytes);
   ALLOC(d.pdf[1], pdf_bytes);
-  // flags padded to whole 32-byte segments (the TMA bulk sweep copies them)
-  const size_t n32 = (size_t)((N + 31) / 32 * 32);
-  ALLOC(d.flags, n32);
+  // flags padded to whole 16-byte words (a lane of the list rebuild reads one)
+  ALLOC(d.flags, (size_t)((N + 31) / 32 * 32));
   ALLOC(d.wallmask, N * sizeof(uint32_t));
   ALLOC(d.phi, N * sizeof(double));
   ALLOC(d.mass, N * sizeof(double));
@@ -745,7 +744,6 @@ fslbm_status fslbm_sync(fslbm_ctx* c) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "fslbm_sync");
   if (herr[0]) return fail(c, FSLBM_EUNSTABLE, "instability: |u|^2 >= c_s^2, rho <= 0 or NaN");
-  if (herr[1]) return fail(c, FSLBM_ETIMEOUT, "a bounded wait for bulk-sweep copies gave up");
   return FSLBM_OK;
 }
 

@@ -33,8 +33,6 @@ inline int iface_coll(const KParams& p) { return coll_of(p) | slip_bit(p); }
 
 template <int Q, class S>
 struct Engine {
-  // the FP32 and 16-bit engines stream the bulk sweep through TMA copies
-  static constexpr bool kTmaBulk = S::kDev && !S::kExactRest && FSLBM_BULK_TMA != 0;
   // persistent bulk blocks per SM the sweep is compiled for
   static constexpr int bulk_blocks_per_sm() {
     return sizeof(typename S::Real) == 4 ? kBulkMinBlocks32 : 2;
@@ -48,7 +46,7 @@ struct Engine {
     return (int)(chunks < cap ? chunks : cap);
   }
   // the FP32 and 16-bit engines fold the geometry pass into the bulk sweep
-  static constexpr bool kFusedGeo = sizeof(typename S::Real) == 4 && !kTmaBulk;
+  static constexpr bool kFusedGeo = sizeof(typename S::Real) == 4;
   // shared-memory carveout (percent of the 228 KB) that holds a tile buffer
   // for every persistent block of the fused sweep; the rest stays L1
   static constexpr int fused_carveout() {
@@ -125,13 +123,7 @@ struct Engine {
     }
     auto bulk = [&](cudaStream_t s2) {
       with_coll(coll, [&](auto C) {
-        constexpr int CO = decltype(C)::value;
-        if constexpr (kTmaBulk && !coll_les(CO)) {
-          constexpr size_t sm = tma_smem<Q, typename S::T>();
-          keep(launch_stage(false, k_bulk_tma<Q, S, CO>, bulk_grid, kBulkBlock, sm, s2, d, p, parity));
-        } else {
-          keep(launch_stage(false, k_bulk<Q, S, CO>, bulk_grid, kBulkBlock, 0, s2, d, p, parity));
-        }
+        keep(launch_stage(false, k_bulk<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, 0, s2, d, p, parity));
       });
     };
     const bool forked = fk && !ev;
@@ -229,15 +221,6 @@ struct Engine {
                          (int)geometry_smem<typename S::Real>());
     cudaFuncSetAttribute(kb_geometry<Q, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)geometry_smem<typename S::Real>());
-    if constexpr (kTmaBulk) {
-      cudaFuncSetAttribute(k_bulk_tma<Q, S, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)tma_smem<Q, typename S::T>());
-      cudaFuncSetAttribute(k_bulk_tma<Q, S, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)tma_smem<Q, typename S::T>());
-      // all persistent blocks resident at once: the most shared memory
-      cudaFuncSetAttribute(k_bulk_tma<Q, S, 0>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      cudaFuncSetAttribute(k_bulk_tma<Q, S, 1>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    }
     Ops o;
     o.init_cells = &init_cells;
     o.init_check = &init_check;
@@ -259,13 +242,8 @@ struct Engine {
         cudaFuncSetAttribute(fns[c], cudaFuncAttributePreferredSharedMemoryCarveout, fused_carveout());
       }
     } else {
-      if constexpr (kTmaBulk) {
-        o.bulk_fn[0] = (const void*)&k_bulk_tma<Q, S, 0>;
-        o.bulk_fn[1] = (const void*)&k_bulk_tma<Q, S, 1>;
-      } else {
-        o.bulk_fn[0] = (const void*)&k_bulk<Q, S, 0>;
-        o.bulk_fn[1] = (const void*)&k_bulk<Q, S, 1>;
-      }
+      o.bulk_fn[0] = (const void*)&k_bulk<Q, S, 0>;
+      o.bulk_fn[1] = (const void*)&k_bulk<Q, S, 1>;
       o.bulk_fn[2] = (const void*)&k_bulk<Q, S, 2>;
       o.bulk_fn[3] = (const void*)&k_bulk<Q, S, 3>;
       o.bulk_fn[4] = (const void*)&k_bulk<Q, S, 4>;
@@ -278,7 +256,7 @@ struct Engine {
     // apply, finalize, list rebuild with the bubbles; while stages are timed
     // the apply stage is two launches when fused and the bubbles are their own
     o.step_launches = kFusedGeo ? 7 : 8;
-    o.bulk_smem = kTmaBulk ? tma_smem<Q, typename S::T>() : kFusedGeo ? geometry_smem<typename S::Real>() : 0;
+    o.bulk_smem = kFusedGeo ? geometry_smem<typename S::Real>() : 0;
     o.batch_step = &batch_step;
     // plan, geometry and bulk sweep (one launch when fused), interface update,
     // resolve, count, apply (two in FP64), finalize,

@@ -24,7 +24,7 @@
 // plain CPU oracle, so results agree to the last bit.
 #pragma once
 
-#include "fslbm_bulk_tma.cuh"
+#include "fslbm_bulk.cuh"
 #include "fslbm_convert.cuh"
 #include "fslbm_interface_lanes.cuh"
 #include <type_traits>
