@@ -186,11 +186,12 @@ __device__ __forceinline__ void bulk_unit(const DPtrs& d, const KParams& p, int 
 // Warps are numbered over the blocks first and from the last block down, so
 // that a short list is spread over the SMs, one unit a warp, and starts on
 // the blocks that hold no geometry tile.
+// FSLBM_BULK_DYN = 0: no hand-out, a fixed stride over the list.
 #ifndef FSLBM_BULK_DYN
 #define FSLBM_BULK_DYN 4
 #endif
 constexpr int kBulkChunk = FSLBM_BULK_DYN;
-static_assert(kBulkChunk >= 1, "the hand-out needs a chunk");
+static_assert(kBulkChunk >= 0, "units a chunk, or 0 for a fixed stride");
 template <class S>
 __host__ __device__ constexpr int short_rounds() {
   return S::kDev && !S::kExactRest ? 4 : 16;
@@ -199,6 +200,10 @@ __host__ __device__ constexpr int short_rounds() {
 template <class S, class F>
 __device__ __forceinline__ void hand_out_units(int n, int* counter, F unit) {
   const int warps = gridDim.x * (kBulkBlock / 32);
+  if constexpr (kBulkChunk == 0) {
+    for (int w = blockIdx.x * (kBulkBlock / 32) + (threadIdx.x >> 5); w < n; w += warps) unit(w);
+    return;
+  }
   constexpr int kShort = short_rounds<S>();
   const int chunk = n >= warps * kShort ? kBulkChunk : 1;
   int base = ((threadIdx.x >> 5) * gridDim.x + (gridDim.x - 1 - blockIdx.x)) * chunk;
