@@ -208,7 +208,7 @@ struct Engine {
 
   static void observables(const DPtrs& d, const KParams& p, int parity, double* out,
                           cudaStream_t st) {
-    k_obs_partial<Q, S, true><<<d.red_blocks, kBlock, 0, st>>>(d, p, parity, d.red);
+    k_obs_partial<Q, S><<<d.red_blocks, kBlock, 0, st>>>(d, p, parity, d.red);
     k_obs_final<<<1, 32 * kObsFields, 0, st>>>(d.red, d.red_blocks, out);
   }
 

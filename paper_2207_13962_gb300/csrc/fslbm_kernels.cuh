@@ -1330,6 +1330,10 @@ static __global__ void __launch_bounds__(kBlock) k_finalize(DPtrs d, KParams p, 
 constexpr int kObsFields = 8;
 constexpr int kObsBlocksPerSm = 4;
 
+__device__ __forceinline__ bool is_nan_bits(double x) {
+  return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+}
+
 // rho - 1 of a cell in FP64, rho in FP32 and the velocity, for the
 // observables (the velocity in post_moments' arithmetic).
 template <int Q, class S>
@@ -1363,9 +1367,7 @@ __device__ __forceinline__ void obs_moments(const typename S::T* P, long long Np
   u[2] = jz / rr - 0.5f * gpar<float>(p, 2);
 }
 
-// kOwn: the state is a context's (liquid cells have fill level 1); otherwise
-// the arrays are a caller's.
-template <int Q, class S, bool kOwn>
+template <int Q, class S>
 __global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d, KParams p, int parity,
                                                                           double* part) {
   using R = typename S::Real;
@@ -1385,12 +1387,13 @@ __global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d
 #pragma unroll
     for (int k = 0; k < 4; ++k) cnt[k] += t == k;
     if (t != T_LIQ && t != T_IFACE) continue;
-    double m = 0.0;
-    if (!kOwn || !S::kDev || t == T_IFACE) {
-      m = d.mass[c];
-      if (!(m == m)) nan = 1;
-    }
-    if (!kOwn || t == T_IFACE) vol += d.phi[c];
+    // mass and fill level of every fluid cell (a checkpoint may hold anything);
+    // a liquid cell's are checked with integer operations and enter the sums
+    // through the count of liquid cells
+    const double m = d.mass[c], ph = d.phi[c];
+    if (is_nan_bits(m)) nan = 1;
+    if (t == T_IFACE) vol += ph;
+    else if (__double_as_longlong(ph) != 0x3ff0000000000000LL) vol += ph - 1.0;
     if constexpr (S::kDev) {
       double dr;
       float rr, u[3];
@@ -1418,7 +1421,7 @@ __global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d
     add_mass(dev);
     add_mass((double)cnt[T_LIQ]);
   }
-  if constexpr (kOwn) vol += (double)cnt[T_LIQ];
+  vol += (double)cnt[T_LIQ];
   __shared__ double sh[kObsFields][kBlock / 32];
   double v[kObsFields] = {mass + mcomp, u2max, vol, (double)nan, (double)cnt[0], (double)cnt[1], (double)cnt[2],
                           (double)cnt[3]};

@@ -95,9 +95,9 @@ extern "C" fslbm_status fslbm_observables_noalloc(const fslbm_domain* domain, in
   double* result = scratch + (size_t)kNoAllocBlocks * kObsFields;
   cudaStream_t st = (cudaStream_t)stream;
   if (q == 19)
-    k_obs_partial<19, StoreF64, false><<<blocks, kBlock, 0, st>>>(d, p, 0, scratch);
+    k_obs_partial<19, StoreF64><<<blocks, kBlock, 0, st>>>(d, p, 0, scratch);
   else
-    k_obs_partial<27, StoreF64, false><<<blocks, kBlock, 0, st>>>(d, p, 0, scratch);
+    k_obs_partial<27, StoreF64><<<blocks, kBlock, 0, st>>>(d, p, 0, scratch);
   k_obs_final<<<1, 32 * kObsFields, 0, st>>>(scratch, blocks, result);
   double h[kObsFields];
   cudaError_t e = cudaGetLastError();
