@@ -145,7 +145,13 @@ typedef struct {
                          Single-domain contexts only (batches reject it). */
 } fslbm_params;
 
-/* Whole-domain observables (FP64 reductions on the device). */
+/* Whole-domain observables, reduced on the device.  The reductions over cells
+ * are in FP64 (masses with a compensated sum per thread).  A liquid cell's rho
+ * is 1 + the sum of its stored PDF deviations: exact in the mass-conserving
+ * formats, within 2^-54 in the other deviation formats (fixed point; a cell
+ * with a deviation of 2 or more: summed in FP64), and an FP64 sum in FSLBM_FP64.
+ * Interface cells count with their FP64 mass.  u is formed in the arithmetic of
+ * the precision, from rho rounded to it once, and |u| in FP64. */
 typedef struct {
   int64_t step;        /* steps done since init                              */
   double total_mass;   /* sum rho (liquid) + sum m (interface), Eq. nm-fslbm-mass */

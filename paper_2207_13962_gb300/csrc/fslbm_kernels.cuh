@@ -1320,13 +1320,15 @@ static __global__ void __launch_bounds__(kBlock) k_finalize(DPtrs d, KParams p, 
 //
 // One read of the PDFs bounds the pass if the FP64 unit (two lanes a clock
 // per SM) is kept out of it, so the deviation formats do their per-cell work
-// in FP32: rho - 1 is summed as a float pair (or in grid steps), u and the
-// candidates for the largest |u| are formed in FP32, and FP64 squares only
-// where the FP32 estimate comes near the largest value so far (the result is
-// the FP64 one).  The mass is the number of liquid cells plus the FP64 sum of
-// their deviations plus the interface masses; |u| is rooted once, at the end.
-// 160x160x512 tube, FP32 (8.2 M fluid cells, 0.65 GB): 1000 us with FP64
-// moments and 2 blocks per SM.
+// in FP32 and integers: rho - 1 is summed in fixed point (see PartSum; grid
+// steps in the mass-conserving formats), u and the candidates for the largest
+// |u| are formed in FP32, and FP64 squares only where the FP32 estimate comes
+// near the largest value so far (the result is the FP64 one).  The mass is the
+// number of liquid cells plus their deviations plus the interface masses; |u|
+// is rooted once, at the end.
+// 160x160x512 tube, FP32 (8.2 M fluid cells, 0.78 GB), a call with the bubble
+// pressures: 1006 us with FP64 moments and 2 blocks per SM, 290 so (284 with
+// float pairs and without the liquid cells' masses and fill levels).
 constexpr int kObsFields = 8;
 constexpr int kObsBlocksPerSm = 4;
 
@@ -1334,11 +1336,49 @@ __device__ __forceinline__ bool is_nan_bits(double x) {
   return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
 }
 
-// rho - 1 of a cell in FP64, rho in FP32 and the velocity, for the
-// observables (the velocity in post_moments' arithmetic).
+// The sum of Q <= 27 floats, |d| < 2, by error-free extraction (Ogita, Rump and
+// Oishi, "Accurate sum and dot product", SIAM J. Sci. Comput. 26, 2005): adding
+// and subtracting 1.5 2^5 rounds d to a multiple of 2^-18, 1.5 2^-15 the rest
+// (at most 2^-19) to one of 2^-38.  h (below 54) and m (below 2^-14) then add
+// up without rounding, and l (terms of at most 2^-39) is within 2^-54 of its
+// sum, so h + m + l is closer to the exact sum than an FP64 sum of 1 + d is.
+// Nine operations a term in three short chains; a float pair by TwoSum takes
+// seven in one chain and loses up to 2^-42 where the terms' exponents differ
+// much.
+struct PartSum {
+  float h = 0.f, m = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float d) {
+    const float a = __fsub_rn(__fadd_rn(48.f, d), 48.f), r = __fsub_rn(d, a);
+    const float b = __fsub_rn(__fadd_rn(0x1.8p-15f, r), 0x1.8p-15f);
+    h = __fadd_rn(h, a);
+    m = __fadd_rn(m, b);
+    l = __fadd_rn(l, __fsub_rn(r, b));
+  }
+  // 1 + the sum, rounded to float once: the rounded sum of the parts, corrected
+  // by what it leaves over (1 + h, the difference and the sum with m are exact)
+  __device__ __forceinline__ float one_plus() const {
+    const float a = __fadd_rn(1.f, h), r = __fadd_rn(a, __fadd_rn(m, l));
+    return __fadd_rn(r, __fadd_rn(__fadd_rn(__fsub_rn(a, r), m), l));
+  }
+};
+
+// rho - 1 summed over cells: multiples of the units below, added as integers.
+// A cell adds less than 2^46 to lo, and a thread of the grid meets fewer than
+// 2^17 cells (a domain has at most 4e8), so neither overflows.
+template <class S>
+struct DevSum {
+  long long hi = 0, lo = 0;
+  __host__ __device__ static constexpr double unit_hi() { return S::kExactRest ? 1.0 / (double)(1LL << grid_shift<S>()) : 0x1p-18; }
+  __host__ __device__ static constexpr double unit_lo() { return 0x1p-60; }
+};
+
+// Adds rho - 1 of a cell to `dev` if add, and gives rho in FP32 and the velocity
+// (in post_moments' arithmetic).  False if the cell's deviations are outside
+// the range of PartSum: then dr is their FP64 sum, and dev is left alone.
 template <int Q, class S>
-__device__ __forceinline__ void obs_moments(const typename S::T* P, long long Np, int c, const KParams& p,
-                                            double& dr, float& rr, float u[3]) {
+__device__ __forceinline__ bool obs_moments(const typename S::T* P, long long Np, int c, const KParams& p, bool add,
+                                            DevSum<S>& dev, double& dr, float& rr, float u[3]) {
+  bool fits = true;
   float f[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) f[i] = load_own<Q, S>(P, Np, c, i);
@@ -1349,22 +1389,34 @@ __device__ __forceinline__ void obs_moments(const typename S::T* P, long long Np
     long long n = n0;
 #pragma unroll
     for (int i = 1; i < Q; ++i) n += grid_steps32<S>(f[i]);  // f[i] is a stored value
-    dr = (double)n * (1.0 / (double)(1LL << S::kShift));
-    rr = d2f(1.0 + dr);
+    rr = d2f(1.0 + (double)n * (1.0 / (double)(1LL << S::kShift)));
+    if (add) dev.hi += n;
   } else {
-    FAcc a;
+    PartSum a;
+    unsigned bits = 0u;  // bit 30 (the exponent's first) is set from 2 on, infinities and NaN included
 #pragma unroll
-    for (int i = 0; i < Q; ++i) a.add(f[i]);
-    dr = a.value();
-    // rho rounded to float, from the pair
-    const float lo = a.lo;
-    a.lo = 0.f;
-    a.add(1.0f);
-    rr = a.hi + (a.lo + lo);
+    for (int i = 0; i < Q; ++i) {
+      a.add(f[i]);
+      bits |= __float_as_uint(f[i]);
+    }
+    fits = !(bits & 0x40000000u);
+    if (fits) {
+      rr = a.one_plus();
+      if (add) {
+        dev.hi += __float2int_rn(a.h * 0x1p18f);
+        dev.lo += ((long long)__float2int_rn(a.m * 0x1p38f) << 22) + __float2int_rn(a.l * 0x1p60f);
+      }
+    } else {
+      dr = 0.0;
+#pragma unroll 1
+      for (int i = 0; i < Q; ++i) dr += (double)load_w<S, Q>(P[(long long)i * Np + c], i);
+      rr = d2f(1.0 + dr);
+    }
   }
   u[0] = jx / rr - 0.5f * gpar<float>(p, 0);
   u[1] = jy / rr - 0.5f * gpar<float>(p, 1);
   u[2] = jz / rr - 0.5f * gpar<float>(p, 2);
+  return fits;
 }
 
 template <int Q, class S>
@@ -1374,7 +1426,8 @@ __global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d
   const typename S::T* P = (const typename S::T*)d.pdf[parity];
   // interface masses (and all masses in FP64) are summed per thread with
   // Neumaier's compensation, then pairwise across threads and blocks
-  double mass = 0.0, mcomp = 0.0, dev = 0.0, u2max = 0.0, vol = 0.0;
+  double mass = 0.0, mcomp = 0.0, u2max = 0.0, vol = 0.0;
+  DevSum<S> dev;  // of the liquid cells (deviation formats)
   float near_max = -1.0f;  // a float bound below the largest |u|^2 so far
   int nan = 0, cnt[4] = {0, 0, 0, 0};
   auto add_mass = [&](double x) {
@@ -1395,9 +1448,9 @@ __global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d
     if (t == T_IFACE) vol += ph;
     else if (__double_as_longlong(ph) != 0x3ff0000000000000LL) vol += ph - 1.0;
     if constexpr (S::kDev) {
-      double dr;
+      double dr = 0.0;
       float rr, u[3];
-      obs_moments<Q, S>(P, p.Np, c, p, dr, rr, u);
+      const bool fits = obs_moments<Q, S>(P, p.Np, c, p, t == T_LIQ, dev, dr, rr, u);
       const float q = __fmaf_rn(u[0], u[0], __fmaf_rn(u[1], u[1], u[2] * u[2]));
       if (!(q == q) || !(rr > 0.0f)) nan = 1;
       if (q >= near_max) {
@@ -1405,8 +1458,8 @@ __global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d
         if (uu > u2max) u2max = uu;
         near_max = (float)u2max * 0.9999f;
       }
-      if (t == T_LIQ) dev += dr;
-      else add_mass(m);
+      if (t == T_IFACE) add_mass(m);
+      else if (!fits) add_mass(dr);
     } else {
       double r;
       R u[3];
@@ -1418,7 +1471,8 @@ __global__ void __launch_bounds__(kBlock, kObsBlocksPerSm) k_obs_partial(DPtrs d
     }
   }
   if constexpr (S::kDev) {
-    add_mass(dev);
+    add_mass((double)dev.hi * dev.unit_hi());
+    add_mass((double)dev.lo * dev.unit_lo());
     add_mass((double)cnt[T_LIQ]);
   }
   vol += (double)cnt[T_LIQ];
