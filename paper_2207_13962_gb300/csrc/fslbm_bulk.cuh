@@ -179,10 +179,19 @@ __device__ __forceinline__ void bulk_unit(const DPtrs& d, const KParams& p, int 
 // in whole chunks it would fill a part of the warps only or leave a last
 // round that is nearly empty, and its sectors stay in L2 anyway.  The line
 // lies where the counter's atomics (one address, so one after another) cost
-// more than that: 4 units a warp for the formats whose units are short, 16
-// where a unit is long (FP64 arithmetic, integer rest sums).  Measured with
-// units against chunks of 4: 96x96x384 tube in FP16SMC (10 units a warp)
-// 101 against 114 us, 192^3 drop in FP32 (5 units a warp) 62.5 against 58.8.
+// more than that: 4 units a warp for the formats whose units are short, 6 for
+// FP32MC, whose units are longer (integer rest sums) but whose sectors leave
+// L2 as FP32's do, 16 where a unit is long and the sectors are half as many or
+// the arithmetic hides them (FP16SMC, FP64).  Step with units one by one /
+// chunks of 4, us (domain, units a warp):
+//   FP32     64x64x256 tube, 2.9: 53.9 / 56.4; 256x128x64 dam, 3.3: 65.1 / 63.7
+//   FP32MC   256x128x64 dam (D3Q27), 4.4: 87 / 92; 192^3 cylinder (D3Q27), 5.6: 113 / 119;
+//            320x160x80 dam, 6.5: 98 / 94; 224^3 drop, 8.1: 122 / 117;
+//            384x192x96 dam, 11: 152 / 114; the same in D3Q27, 15: 210 / 164
+//   FP16SMC  256x128x64 dam (D3Q27), 4.4: 86 / 92; 320x160x80 dam, 6.5: 98 / 101;
+//            96x96x384 tube, 10: 118 / 121; 256^3 cylinder (D3Q27), 15: 215 / 214
+//   FP64     192^3 cylinder (D3Q27), 8.4: 1090 / 1145; 192^3 drop, 10: 962 / 981;
+//            208^3 cylinder (D3Q27), 13: 1643 / 1636
 // Warps are numbered over the blocks first and from the last block down, so
 // that a short list is spread over the SMs, one unit a warp, and starts on
 // the blocks that hold no geometry tile.
@@ -194,7 +203,7 @@ constexpr int kBulkChunk = FSLBM_BULK_DYN;
 static_assert(kBulkChunk >= 0, "units a chunk, or 0 for a fixed stride");
 template <class S>
 __host__ __device__ constexpr int short_rounds() {
-  return S::kDev && !S::kExactRest ? 4 : 16;
+  return !S::kDev ? 16 : !S::kExactRest ? 4 : sizeof(typename S::T) == 4 ? 6 : 16;
 }
 
 template <class S, class F>
@@ -219,9 +228,11 @@ __device__ __forceinline__ void hand_out_units(int n, int* counter, F unit) {
 // Resident blocks per SM a bulk sweep is compiled for: the FP32 engines
 // kBulkMinBlocks32 (64 registers), 3 with the Smagorinsky model (its
 // momentum flux needs more) and in the mass-conserving formats with 27
-// directions (8 cylinders in FP16SMC, a step: 128 us, 131 with four blocks;
-// with 19 directions three lose, 96x96x384 tube 121 against 115), the FP64
-// engine 2.
+// directions, the FP64 engine 2.  Step with three / four blocks, us: D3Q27
+// FP16SMC, 8 cylinders in a batch 128 / 131; D3Q27 FP32MC, 160x160x384 tube
+// 298 / 304, 8 cylinders in a batch 274 / 280; D3Q27 FP32, the same tube 272 /
+// 264, cylinders 246 / 244; D3Q19 FP16SMC, the tube 239 / 227, 8 drops in a
+// batch 326 / 320; D3Q19 FP32MC 224 / 209 and 313 / 306.
 template <int Q, class S, int COLL>
 constexpr int bulk_min_blocks() {
   return sizeof(typename S::Real) == 4 ? (coll_les(COLL) || (S::kExactRest && Q == 27) ? 3 : kBulkMinBlocks32) : 2;
