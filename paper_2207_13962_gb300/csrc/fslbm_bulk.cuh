@@ -17,8 +17,7 @@ namespace fslbm {
 // is race-free, and next step x pulls its bounced-back PDF from the constant
 // offset like any interior cell: the bulk sweep reads at constant offsets
 // except next to a non-periodic domain face (own-slot bounce-back) or across
-// a periodic face (wrapped index), which take the general path.  Every
-// kernel that produces post-collision PDFs of a fluid cell (bulk, interface,
+// a periodic face (wrap distances; see below).  Every kernel that produces post-collision PDFs of a fluid cell (bulk, interface,
 // new interface cells, init) writes these reflected copies.
 constexpr int kBulkBlock = 256;
 
@@ -67,8 +66,7 @@ __device__ __forceinline__ Wraps wraps_at(const KParams& p, int x, int y, int z)
   return w;
 }
 
-// One liquid cell, loads straight from global memory (storage formats of
-// 2 bytes, and batches).
+// One liquid cell, loads straight from global memory.
 template <int Q, class S, int COLL>
 __device__ __forceinline__ void bulk_cell(const DPtrs& d, const KParams& p, int parity, int c,
                                           uint8_t fl, int path) {
@@ -78,7 +76,7 @@ __device__ __forceinline__ void bulk_cell(const DPtrs& d, const KParams& p, int 
   T* __restrict__ B = (T*)d.pdf[parity ^ 1];
   const long long Np = p.Np;
   R f[Q];
-  // the mass-conserving formats hold the rest PDF in an FP64 slice
+  // the mass-conserving formats hold the rest PDF in an int32 slice
   constexpr int i0 = S::kExactRest ? 1 : 0;
   if (path == kInterior) {
     const T* Ac = A + c;
@@ -90,7 +88,7 @@ __device__ __forceinline__ void bulk_cell(const DPtrs& d, const KParams& p, int 
     if constexpr (coll_slip(COLL)) {
 #pragma unroll
       for (int i = i0; i < Q; ++i)
-        f[i] = load_w<S, Q>(A[pull_index_general<Q, true>(p, d.flags, c, x, y, z, i)], i);
+        f[i] = load_w<S, Q>(A[pull_index_slip<Q>(p, d.flags, c, x, y, z, i)], i);
     } else {
       // a bit per no-slip face the cell touches, tested against the faces a
       // direction is pulled through

@@ -50,9 +50,6 @@ __device__ __forceinline__ int nbr(const KParams& p, int x, int y, int z, int dx
   if (X < 0 || Y < 0 || Z < 0) return -1;
   return cidx(p, X, Y, Z);
 }
-__device__ __forceinline__ int ntype(const uint8_t* flags, int n) {
-  return n < 0 ? T_OBST : (flags[n] & F_TYPE);
-}
 
 // warp-aggregated append; every lane of the warp must call it
 __device__ __forceinline__ int warp_append(int* counter, bool pred) {
@@ -675,38 +672,19 @@ __device__ __forceinline__ int pull_source(const KParams& p, int x, int y, int z
   return out ? -1 : cidx(p, X, Y, Z);
 }
 
-// Index (slice and cell) of the value a liquid cell c at (x, y, z) pulls in
-// direction i: its source's PDF (wrapped across periodic faces; with SLIP,
-// reflected at free-slip faces), or its own PDF ibar (bounce-back) when the
-// source lies across a no-slip face or the mirror image across a free-slip
-// face is an obstacle cell.  Without SLIP the free-slip logic is not
-// compiled (domains without free-slip faces).
-template <int Q, bool SLIP>
-__device__ __forceinline__ long long pull_index_general(const KParams& p, const uint8_t* flags, int c,
-                                                        int x, int y, int z, int i) {
-  if constexpr (SLIP) {
-    int j;
-    bool mir;
-    const int s = pull_source<Q>(p, x, y, z, i, j, mir);
-    if (s < 0 || (mir && (flags[s] & F_TYPE) == T_OBST)) return (long long)OPP(i) * p.Np + c;
-    return (long long)j * p.Np + s;
-  } else {
-    int X = x - CX(i), Y = y - CY(i), Z = z - CZ(i);
-    bool out = false;
-    if (X < 0 || X >= p.nx) {
-      if (p.per[0]) X = X < 0 ? X + p.nx : X - p.nx;
-      else out = true;
-    }
-    if (Y < 0 || Y >= p.ny) {
-      if (p.per[1]) Y = Y < 0 ? Y + p.ny : Y - p.ny;
-      else out = true;
-    }
-    if (Z < 0 || Z >= p.nz) {
-      if (p.per[2]) Z = Z < 0 ? Z + p.nz : Z - p.nz;
-      else out = true;
-    }
-    return out ? (long long)OPP(i) * p.Np + c : (long long)i * p.Np + cidx(p, X, Y, Z);
-  }
+// Index (slice and cell) of the value a liquid cell c at (x, y, z) of a domain
+// with free-slip faces pulls in direction i: its source's PDF (wrapped across
+// periodic faces, reflected at free-slip faces), or its own PDF ibar
+// (bounce-back) when the source lies across a no-slip face or the mirror image
+// across a free-slip face is an obstacle cell.
+template <int Q>
+__device__ __forceinline__ long long pull_index_slip(const KParams& p, const uint8_t* flags, int c,
+                                                     int x, int y, int z, int i) {
+  int j;
+  bool mir;
+  const int s = pull_source<Q>(p, x, y, z, i, j, mir);
+  if (s < 0 || (mir && (flags[s] & F_TYPE) == T_OBST)) return (long long)OPP(i) * p.Np + c;
+  return (long long)j * p.Np + s;
 }
 
 // Slot of the obstacle pull source x - c_i (inside the domain or across a

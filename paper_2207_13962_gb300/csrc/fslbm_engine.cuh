@@ -119,40 +119,40 @@ struct Engine {
       if (ev) ev->mark(6, st);
       keep(launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity));
       list_and_bubbles();
-      return keep.e;
-    }
-    auto bulk = [&](cudaStream_t s2) {
+    } else {
+      auto bulk = [&](cudaStream_t s2) {
+        with_coll(coll, [&](auto C) {
+          keep(launch_stage(false, k_bulk<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, 0, s2, d, p, parity));
+        });
+      };
+      const bool forked = fk && !ev;
+      auto fork_bulk = [&]() {
+        keep(cudaEventRecord(fk->fork, st));
+        keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
+        bulk(fk->side);
+        keep(cudaEventRecord(fk->join, fk->side));
+      };
+      if (ev) ev->mark(0, st);
+      if (forked) fork_bulk();
+      keep(launch_stage(false, k_geometry<Q, S>, band_grid * kGeoGridMult, kGeoBlock,
+                        geometry_smem<typename S::Real>(), st, d, p, parity));
+      if (ev) ev->mark(1, st);
+      if (!forked) bulk(st);
+      if (ev) ev->mark(2, st);
       with_coll(coll, [&](auto C) {
-        keep(launch_stage(false, k_bulk<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, 0, s2, d, p, parity));
+        keep(launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity));
       });
-    };
-    const bool forked = fk && !ev;
-    auto fork_bulk = [&]() {
-      keep(cudaEventRecord(fk->fork, st));
-      keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
-      bulk(fk->side);
-      keep(cudaEventRecord(fk->join, fk->side));
-    };
-    if (ev) ev->mark(0, st);
-    if (forked) fork_bulk();
-    keep(launch_stage(false, k_geometry<Q, S>, band_grid * kGeoGridMult, kGeoBlock,
-                      geometry_smem<typename S::Real>(), st, d, p, parity));
-    if (ev) ev->mark(1, st);
-    if (!forked) bulk(st);
-    if (ev) ev->mark(2, st);
-    with_coll(coll, [&](auto C) {
-      keep(launch_stage(chained, k_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, d, p, parity));
-    });
-    if (ev) ev->mark(3, st);
-    keep(launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity));
-    if (ev) ev->mark(4, st);
-    keep(launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity));
-    if (ev) ev->mark(5, st);
-    if (forked) keep(cudaStreamWaitEvent(st, fk->join, 0));
-    keep(launch_stage(chained && !forked, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity));
-    if (ev) ev->mark(6, st);
-    keep(launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity));
-    list_and_bubbles();
+      if (ev) ev->mark(3, st);
+      keep(launch_stage(chained, k_resolve<Q>, band_grid * 2, kBlock, 0, st, d, p, parity));
+      if (ev) ev->mark(4, st);
+      keep(launch_stage(chained, k_count<Q, S>, band_grid * 2, kBlock, 0, st, d, p, parity));
+      if (ev) ev->mark(5, st);
+      if (forked) keep(cudaStreamWaitEvent(st, fk->join, 0));
+      keep(launch_stage(chained && !forked, k_apply<Q, S, true, true>, band_grid * 2, kBlock, 0, st, d, p, parity));
+      if (ev) ev->mark(6, st);
+      keep(launch_stage(chained, k_finalize, band_grid, kBlock, 0, st, d, p, parity));
+      list_and_bubbles();
+    }
     return keep.e;
   }
 
@@ -179,31 +179,31 @@ struct Engine {
       keep(launch_stage(true, kb_finalize, band_grid, kBlock, 0, st, recs, pl));
       keep(launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs));
       (void)fk;
-      return keep.e;
+    } else {
+      keep(cudaEventRecord(fk->fork, st));
+      keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
+      with_coll(collision, [&](auto C) {
+        keep(launch_stage(false, kb_bulk<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, 0, fk->side, recs, pl));
+      });
+      keep(cudaEventRecord(fk->join, fk->side));
+      keep(launch_stage(false, kb_geometry<Q, S>, band_grid * kGeoGridMult, kGeoBlock, sm, st, recs, pl));
+      with_coll(collision, [&](auto C) {
+        keep(launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl));
+      });
+      keep(launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl));
+      keep(launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl));
+      keep(cudaStreamWaitEvent(st, fk->join, 0));
+      // the new cells' FP64 chains beside the receivers' (4 drops of 48 to 80
+      // cells a side: 315.2 us a step so, 315.4 in one launch)
+      keep(cudaEventRecord(fk->fork, st));
+      keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
+      keep(launch_stage(false, kb_apply<Q, S, true, false>, band_grid * 2, kBlock, 0, fk->side, recs, pl));
+      keep(cudaEventRecord(fk->join, fk->side));
+      keep(launch_stage(false, kb_apply<Q, S, false, true>, band_grid * 2, kBlock, 0, st, recs, pl));
+      keep(cudaStreamWaitEvent(st, fk->join, 0));
+      keep(launch_stage(false, kb_finalize, band_grid, kBlock, 0, st, recs, pl));
+      keep(launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs));
     }
-    keep(cudaEventRecord(fk->fork, st));
-    keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
-    with_coll(collision, [&](auto C) {
-      keep(launch_stage(false, kb_bulk<Q, S, decltype(C)::value>, bulk_grid, kBulkBlock, 0, fk->side, recs, pl));
-    });
-    keep(cudaEventRecord(fk->join, fk->side));
-    keep(launch_stage(false, kb_geometry<Q, S>, band_grid * kGeoGridMult, kGeoBlock, sm, st, recs, pl));
-    with_coll(collision, [&](auto C) {
-      keep(launch_stage(true, kb_interface<Q, S, decltype(C)::value>, band_grid * 2, 128, 0, st, recs, pl));
-    });
-    keep(launch_stage(true, kb_resolve<Q>, band_grid * 2, kBlock, 0, st, recs, pl));
-    keep(launch_stage(true, kb_count<Q, S>, band_grid * 2, kBlock, 0, st, recs, pl));
-    keep(cudaStreamWaitEvent(st, fk->join, 0));
-    // the new cells' FP64 chains beside the receivers' (4 drops of 48 to 80
-    // cells a side: 315.2 us a step so, 315.4 in one launch)
-    keep(cudaEventRecord(fk->fork, st));
-    keep(cudaStreamWaitEvent(fk->side, fk->fork, 0));
-    keep(launch_stage(false, kb_apply<Q, S, true, false>, band_grid * 2, kBlock, 0, fk->side, recs, pl));
-    keep(cudaEventRecord(fk->join, fk->side));
-    keep(launch_stage(false, kb_apply<Q, S, false, true>, band_grid * 2, kBlock, 0, st, recs, pl));
-    keep(cudaStreamWaitEvent(st, fk->join, 0));
-    keep(launch_stage(false, kb_finalize, band_grid, kBlock, 0, st, recs, pl));
-    keep(launch_stage(true, kb_bubble_end, pl.n, 256, 0, st, recs));
     return keep.e;
   }
 
@@ -218,10 +218,12 @@ struct Engine {
   }
 
   static Ops ops() {
-    cudaFuncSetAttribute(k_geometry<Q, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)geometry_smem<typename S::Real>());
-    cudaFuncSetAttribute(kb_geometry<Q, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)geometry_smem<typename S::Real>());
+    if constexpr (!kFusedGeo) {
+      cudaFuncSetAttribute(k_geometry<Q, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)geometry_smem<typename S::Real>());
+      cudaFuncSetAttribute(kb_geometry<Q, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)geometry_smem<typename S::Real>());
+    }
     Ops o;
     o.init_cells = &init_cells;
     o.init_check = &init_check;
@@ -243,14 +245,14 @@ struct Engine {
         cudaFuncSetAttribute(fns[c], cudaFuncAttributePreferredSharedMemoryCarveout, fused_carveout());
       }
     } else {
-      o.bulk_fn[0] = (const void*)&k_bulk<Q, S, 0>;
-      o.bulk_fn[1] = (const void*)&k_bulk<Q, S, 1>;
-      o.bulk_fn[2] = (const void*)&k_bulk<Q, S, 2>;
-      o.bulk_fn[3] = (const void*)&k_bulk<Q, S, 3>;
-      o.bulk_fn[4] = (const void*)&k_bulk<Q, S, 4>;
-      o.bulk_fn[5] = (const void*)&k_bulk<Q, S, 5>;
-      o.bulk_fn[6] = (const void*)&k_bulk<Q, S, 6>;
-      o.bulk_fn[7] = (const void*)&k_bulk<Q, S, 7>;
+        o.bulk_fn[0] = (const void*)&k_bulk<Q, S, 0>;
+        o.bulk_fn[1] = (const void*)&k_bulk<Q, S, 1>;
+        o.bulk_fn[2] = (const void*)&k_bulk<Q, S, 2>;
+        o.bulk_fn[3] = (const void*)&k_bulk<Q, S, 3>;
+        o.bulk_fn[4] = (const void*)&k_bulk<Q, S, 4>;
+        o.bulk_fn[5] = (const void*)&k_bulk<Q, S, 5>;
+        o.bulk_fn[6] = (const void*)&k_bulk<Q, S, 6>;
+        o.bulk_fn[7] = (const void*)&k_bulk<Q, S, 7>;
     }
     o.bulk_blocks_per_sm = bulk_blocks_per_sm();
     // bulk and geometry (one launch when fused), interface, resolve, count,
@@ -273,14 +275,14 @@ struct Engine {
         cudaFuncSetAttribute(fns[c], cudaFuncAttributePreferredSharedMemoryCarveout, fused_carveout());
       }
     } else {
-      o.batch_bulk_fn[0] = (const void*)&kb_bulk<Q, S, 0>;
-      o.batch_bulk_fn[1] = (const void*)&kb_bulk<Q, S, 1>;
-      o.batch_bulk_fn[2] = (const void*)&kb_bulk<Q, S, 2>;
-      o.batch_bulk_fn[3] = (const void*)&kb_bulk<Q, S, 3>;
-      o.batch_bulk_fn[4] = (const void*)&kb_bulk<Q, S, 4>;
-      o.batch_bulk_fn[5] = (const void*)&kb_bulk<Q, S, 5>;
-      o.batch_bulk_fn[6] = (const void*)&kb_bulk<Q, S, 6>;
-      o.batch_bulk_fn[7] = (const void*)&kb_bulk<Q, S, 7>;
+        o.batch_bulk_fn[0] = (const void*)&kb_bulk<Q, S, 0>;
+        o.batch_bulk_fn[1] = (const void*)&kb_bulk<Q, S, 1>;
+        o.batch_bulk_fn[2] = (const void*)&kb_bulk<Q, S, 2>;
+        o.batch_bulk_fn[3] = (const void*)&kb_bulk<Q, S, 3>;
+        o.batch_bulk_fn[4] = (const void*)&kb_bulk<Q, S, 4>;
+        o.batch_bulk_fn[5] = (const void*)&kb_bulk<Q, S, 5>;
+        o.batch_bulk_fn[6] = (const void*)&kb_bulk<Q, S, 6>;
+        o.batch_bulk_fn[7] = (const void*)&kb_bulk<Q, S, 7>;
     }
     return o;
   }

@@ -831,7 +831,8 @@ __device__ __forceinline__ void hand_out_tiles(int n, int* counter, int* s_tile,
 // Taylor bubble: separate kernels 77.5 + 295 us, every block first on tiles
 // 345 us, every second block 364 us, every fourth 361 us: the sweep needs all
 // its blocks to keep HBM busy, so blocks held by tiles slow it by about what
-// running the tiles beside it saves.
+// running the tiles beside it saves.  (Figures of when a tile took twice as
+// long; the launch takes 326 to 330 us now.)
 template <int Q, class S, int COLL>
 __global__ void __launch_bounds__(kBulkBlock, (bulk_min_blocks<Q, S, COLL>()))
     k_bulk_geo(DPtrs d, KParams p, int parity) {
