@@ -240,7 +240,7 @@ fslbm_status fslbm_create(const fslbm_domain* domain, fslbm_lattice lattice,
   if (e == cudaSuccess) e = dalloc(c, &(ptr), (bytes));
   ALLOC(d.pdf[0], pdf_bytes);
   ALLOC(d.pdf[1], pdf_bytes);
-  // flags padded to whole 16-byte words (a lane of the list rebuild reads one)
+  // flags padded to whole 32-byte sectors
   ALLOC(d.flags, (size_t)((N + 31) / 32 * 32));
   ALLOC(d.wallmask, N * sizeof(uint32_t));
   ALLOC(d.phi, N * sizeof(double));
